@@ -30,45 +30,15 @@ __device__ __forceinline__ bool tile_active(const LayerArgs& a, const Tile& t, i
     return tile_active_g(a, t, a.gl, k);
 }
 
-// ----------------------------------------------------------------------------------
-// Epilogue on one row segment of 16 columns (shared logic of the centred update).
-// ----------------------------------------------------------------------------------
-__device__ __forceinline__ void store_operand(int fmt, uint8_t* base, size_t plane, size_t idx, float zs) {
-    switch (fmt) {
-        case OP_F32:
-            reinterpret_cast<float*>(base)[idx] = zs;
-            break;
-        case OP_TF32X3: {
-            uint32_t hb;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hb) : "f"(zs));
-            const float h = __uint_as_float(hb);
-            uint32_t lb;   // low part rounded to the TF32 bits the tensor core reads
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lb) : "f"(zs - h));
-            reinterpret_cast<float*>(base)[idx] = h;
-            reinterpret_cast<float*>(base)[plane + idx] = __uint_as_float(lb);
-            break;
-        }
-        case OP_BF16X3: {
-            const __nv_bfloat16 b0 = __float2bfloat16_rn(zs);
-            const float r1 = zs - __bfloat162float(b0);
-            const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 b2 = __float2bfloat16_rn(r1 - __bfloat162float(b1));
-            __nv_bfloat16* p = reinterpret_cast<__nv_bfloat16*>(base);
-            p[idx] = b0;
-            p[plane + idx] = b1;
-            p[2 * plane + idx] = b2;
-            break;
-        }
-        case OP_F16X2: {
-            const __half h = __float2half_rn(zs);
-            const __half l = __float2half_rn(zs - __half2float(h));
-            __half* p = reinterpret_cast<__half*>(base);
-            p[idx] = h;
-            p[plane + idx] = l;
-            break;
-        }
-    }
+// 16-byte asynchronous global -> shared copies through the load/store path
+// (cp.async, L2 only).  The store warps of the tensor-core kernel use them so
+// that their loads do not queue behind the operand tiles in the TMA unit.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 struct EpiCtx {
     int n, P, chain, kind, flip, last, next_fmt;
@@ -79,71 +49,86 @@ struct EpiCtx {
     double cdiag;         // f0 (or 1 - f0 when flipped) added on the diagonal of D
 };
 
-// Process row r, columns c0 .. c0 + W - 1 (c0 % 8 == 0, W % 4 == 0, c0 + W <= P) with
-// accumulator values v[W].  Accumulates (diagonal sum, weighted square sum) of the
-// centred output G into tr / sq at the last layer.
-template <int W>
-__device__ __forceinline__ void epi_segment(const LayerArgs& a, const EpiCtx& e, int r, int c0,
-                                            const float* v, double& tr, double& sq) {
-    if (r >= e.n) return;
-    float* Zs = a.Z[e.chain] + e.slab;
-    float* As = a.A[e.chain] + e.slab;
-    float z[W], ac[W];
-#pragma unroll
-    for (int i = 0; i < W / 4; ++i) {
-        const size_t o = state_off(e.P, r, c0 + 4 * i);
-        const float4 zz = *reinterpret_cast<const float4*>(Zs + o);
-        const float4 aa = *reinterpret_cast<const float4*>(As + o);
-        z[4 * i + 0] = zz.x; z[4 * i + 1] = zz.y; z[4 * i + 2] = zz.z; z[4 * i + 3] = zz.w;
-        ac[4 * i + 0] = aa.x; ac[4 * i + 1] = aa.y; ac[4 * i + 2] = aa.z; ac[4 * i + 3] = aa.w;
-    }
-    float zn[W], an[W];
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-        const float xh = fmaf(e.mul, v[j], e.L.bp * z[j]);
-        an[j] = fmaf(e.L.d2, xh, fmaf(e.L.d, z[j], ac[j]));
-        zn[j] = e.last ? xh : fmaf(e.L.p, xh, e.L.q * ac[j]);
-    }
-    if (!e.last) {
-#pragma unroll
-        for (int i = 0; i < W / 4; ++i) {
-            const size_t o = state_off(e.P, r, c0 + 4 * i);
-            *reinterpret_cast<float4*>(Zs + o) = make_float4(zn[4 * i], zn[4 * i + 1], zn[4 * i + 2], zn[4 * i + 3]);
-            *reinterpret_cast<float4*>(As + o) = make_float4(an[4 * i], an[4 * i + 1], an[4 * i + 2], an[4 * i + 3]);
-        }
-        uint8_t* ob = a.opw[e.chain];
-        const float os = e.next_fmt == OP_F16X2 ? e.L.out_scale : 1.f;
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const int c = c0 + j;
-            if (c < e.n && r <= c) {
-                const float zs = zn[j] * os;
-                store_operand(e.next_fmt, ob, a.plane_elems, e.slab + (size_t)r * e.P + c, zs);
-                if (c != r) store_operand(e.next_fmt, ob, a.plane_elems, e.slab + (size_t)c * e.P + r, zs);
-            }
-        }
+// CUDA-core epilogues: row r, columns c0 .. c0 + 7 (c0 % 8 == 0) with the
+// products v, one row per lane of a 32-row block.  The next layer's operands
+// are the full FP32 matrix: the direct row as two 16-byte vectors when all of
+// it lies in the triangle and the order, the mirror (c, r) one element per
+// lane, a contiguous run of row c across the warp.
+__device__ __forceinline__ void store_operands8(const LayerArgs& a, const EpiCtx& e, int r, int c0, const float* z) {
+    float* const op = reinterpret_cast<float*>(a.opw[e.chain]) + e.slab;
+    float* const row = op + (size_t)r * e.P + c0;
+    if (r <= c0 && c0 + 7 < e.n) {
+        reinterpret_cast<float4*>(row)[0] = make_float4(z[0], z[1], z[2], z[3]);
+        reinterpret_cast<float4*>(row)[1] = make_float4(z[4], z[5], z[6], z[7]);
     } else {
 #pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const int c = c0 + j;
-            if (c < e.n && r <= c) {
-                const float g = fmaf(e.L.g, zn[j], an[j]);
-                if (e.kind == CHAIN_FERMI && a.D) {
-                    float dv;
-                    if (e.flip) dv = (r == c ? (float)e.cdiag : 0.f) - g;
-                    else dv = g + (r == c ? (float)e.cdiag : 0.f);
-                    a.D[e.doff + (int64_t)r * e.n + c] = dv;
-                    if (c != r) a.D[e.doff + (int64_t)c * e.n + r] = dv;
-                }
-                const double gd = (double)g;
-                if (r == c) {
-                    tr += gd;
-                    sq += gd * gd;
-                } else {
-                    sq += 2.0 * gd * gd;
-                }
+        for (int j = 0; j < 8; ++j)
+            if (c0 + j < e.n && r <= c0 + j) row[j] = z[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (c0 + j < e.n && r < c0 + j) op[(size_t)(c0 + j) * e.P + r] = z[j];
+}
+
+// Last layer: D from the centred output g (Fermi chain) and the (diagonal sum,
+// weighted square sum) of g in FP64.
+__device__ __forceinline__ void store_last8(const LayerArgs& a, const EpiCtx& e, int r, int c0, const float* g,
+                                            double& tr, double& sq) {
+    const bool dout = e.kind == CHAIN_FERMI && a.D;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int c = c0 + j;
+        if (c < e.n && r <= c) {
+            if (dout) {
+                float dv;
+                if (e.flip) dv = (r == c ? (float)e.cdiag : 0.f) - g[j];
+                else dv = g[j] + (r == c ? (float)e.cdiag : 0.f);
+                a.D[e.doff + (int64_t)r * e.n + c] = dv;
+                if (c != r) a.D[e.doff + (int64_t)c * e.n + r] = dv;
+            }
+            const double gd = (double)g[j];
+            if (r == c) {
+                tr += gd;
+                sq += gd * gd;
+            } else {
+                sq += 2.0 * gd * gd;
             }
         }
+    }
+}
+
+// The 8 state values of row r, columns c0 .. c0 + 7 (two float4 runs 128 floats
+// apart in the blocked layout).
+__device__ __forceinline__ void load_state8(const float* S, float* x) {
+    const float4 u = reinterpret_cast<const float4*>(S)[0], w = reinterpret_cast<const float4*>(S + 128)[0];
+    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = w.x; x[5] = w.y; x[6] = w.z; x[7] = w.w;
+}
+__device__ __forceinline__ void store_state8(float* S, const float* x) {
+    reinterpret_cast<float4*>(S)[0] = make_float4(x[0], x[1], x[2], x[3]);
+    reinterpret_cast<float4*>(S + 128)[0] = make_float4(x[4], x[5], x[6], x[7]);
+}
+
+__device__ __forceinline__ void epi_segment(const LayerArgs& a, const EpiCtx& e, int r, int c0, const float* v,
+                                            double& tr, double& sq) {
+    if (r >= e.n) return;
+    const size_t so = e.slab + state_off(e.P, r, c0);
+    float* const Zs = a.Z[e.chain] + so;
+    float* const As = a.A[e.chain] + so;
+    float z[8], ac[8], zn[8], an[8];
+    load_state8(Zs, z);
+    load_state8(As, ac);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float xh = fmaf(e.mul, v[j], e.L.bp * z[j]);
+        an[j] = fmaf(e.L.d2, xh, fmaf(e.L.d, z[j], ac[j]));
+        zn[j] = e.last ? fmaf(e.L.g, xh, an[j]) : fmaf(e.L.p, xh, e.L.q * ac[j]);
+    }
+    if (!e.last) {
+        store_state8(Zs, zn);
+        store_state8(As, an);
+        store_operands8(a, e, r, c0, zn);
+    } else {
+        store_last8(a, e, r, c0, zn, tr, sq);
     }
 }
 
@@ -158,76 +143,40 @@ __device__ __forceinline__ void epi_segment(const LayerArgs& a, const EpiCtx& e,
 // the last layer forms G = sum_{j<=L} gamma_j x^_j instead (D = G + f0 I).
 // U^_k is re-formed here from the planes in the order its operands were
 // formed, so it equals the operand value the product used.
-template <int W>
-__device__ __forceinline__ void epi_segment_max(const LayerArgs& a, const EpiCtx& e, int r, int c0,
-                                                const float* v, double& tr, double& sq) {
+__device__ __forceinline__ void epi_segment_max(const LayerArgs& a, const EpiCtx& e, int r, int c0, const float* v,
+                                                double& tr, double& sq) {
     if (r >= e.n) return;
-    float* X = a.Z[e.chain] + e.slab;
+    float* const X = a.Z[e.chain] + e.slab + state_off(e.P, r, c0);
     const int k1 = e.L.nplanes;                    // k + 1 stored layers are read
     const float* th = a.coef + e.L.coef;           // theta_{k,0..k}
     const float* tn = th + k1;                     // theta_{k+1,0..k+1}
     const float* gm = tn + k1 + 1;                 // gamma_{0..L} (last layer)
-    float ui[W], un[W], g[W];
+    float ui[8], un[8];                            // un: U^_{k+1} so far, or G at the last layer
 #pragma unroll
-    for (int j = 0; j < W; ++j) ui[j] = un[j] = g[j] = 0.f;
+    for (int j = 0; j < 8; ++j) ui[j] = un[j] = 0.f;
+#pragma unroll 4
     for (int p = 0; p < k1; ++p) {
-        const float tk = th[p], tq = tn[p], gp = e.last ? gm[p] : 0.f;
-        const float* Xp = X + (size_t)p * a.plane_elems;
+        const float tk = th[p], tq = e.last ? gm[p] : tn[p];
+        float x[8];
+        load_state8(X + (size_t)p * a.plane_elems, x);
 #pragma unroll
-        for (int i = 0; i < W / 4; ++i) {
-            const float4 xx = *reinterpret_cast<const float4*>(Xp + state_off(e.P, r, c0 + 4 * i));
-            const float xv[4] = {xx.x, xx.y, xx.z, xx.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                ui[4 * i + q] = fmaf(tk, xv[q], ui[4 * i + q]);
-                un[4 * i + q] = fmaf(tq, xv[q], un[4 * i + q]);
-                g[4 * i + q] = fmaf(gp, xv[q], g[4 * i + q]);
-            }
+        for (int j = 0; j < 8; ++j) {
+            ui[j] = fmaf(tk, x[j], ui[j]);
+            un[j] = fmaf(tq, x[j], un[j]);
         }
     }
-    float xn[W];
+    float xn[8];
+    const float tl = e.last ? gm[k1] : tn[k1];
 #pragma unroll
-    for (int j = 0; j < W; ++j) xn[j] = fmaf(e.mul, v[j], e.L.bp * ui[j]);
+    for (int j = 0; j < 8; ++j) {
+        xn[j] = fmaf(e.mul, v[j], e.L.bp * ui[j]);
+        un[j] = fmaf(tl, xn[j], un[j]);
+    }
     if (!e.last) {
-        float* Xn = X + (size_t)k1 * a.plane_elems;
-#pragma unroll
-        for (int i = 0; i < W / 4; ++i)
-            *reinterpret_cast<float4*>(Xn + state_off(e.P, r, c0 + 4 * i)) =
-                make_float4(xn[4 * i], xn[4 * i + 1], xn[4 * i + 2], xn[4 * i + 3]);
-        const float tl = tn[k1];
-        uint8_t* ob = a.opw[e.chain];
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const int c = c0 + j;
-            if (c < e.n && r <= c) {
-                const float zs = fmaf(tl, xn[j], un[j]);
-                store_operand(e.next_fmt, ob, a.plane_elems, e.slab + (size_t)r * e.P + c, zs);
-                if (c != r) store_operand(e.next_fmt, ob, a.plane_elems, e.slab + (size_t)c * e.P + r, zs);
-            }
-        }
+        store_state8(X + (size_t)k1 * a.plane_elems, xn);
+        store_operands8(a, e, r, c0, un);
     } else {
-        const float gl = gm[k1];
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const int c = c0 + j;
-            if (c < e.n && r <= c) {
-                const float gv = fmaf(gl, xn[j], g[j]);
-                if (e.kind == CHAIN_FERMI && a.D) {
-                    float dv;
-                    if (e.flip) dv = (r == c ? (float)e.cdiag : 0.f) - gv;
-                    else dv = gv + (r == c ? (float)e.cdiag : 0.f);
-                    a.D[e.doff + (int64_t)r * e.n + c] = dv;
-                    if (c != r) a.D[e.doff + (int64_t)c * e.n + r] = dv;
-                }
-                const double gd = (double)gv;
-                if (r == c) {
-                    tr += gd;
-                    sq += gd * gd;
-                } else {
-                    sq += 2.0 * gd * gd;
-                }
-            }
-        }
+        store_last8(a, e, r, c0, un, tr, sq);
     }
 }
 

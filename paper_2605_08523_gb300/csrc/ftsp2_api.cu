@@ -830,8 +830,7 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
             const bool use_ref = !all_simt;
             la.tiles = use_ref ? tiles_ref : tiles;
             la.ntiles = use_ref ? L.ntiles_ref : L.ntiles;
-            const int grid = std::max(1, std::min(la.ntiles, di.sms * 4));
-            e = launch_layer_simt(la, grid, s);
+            e = launch_layer_simt(la, s);
             last_table = use_ref ? 1 : 0;
         } else {
             la.tiles = pair ? tiles : tiles_ref;

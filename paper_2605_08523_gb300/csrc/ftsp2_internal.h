@@ -283,8 +283,8 @@ cudaError_t launch_layer_tc(int mode, const LayerArgs& a, const TmaMaps& maps, c
 // can be resident at once (0 if unknown): the bound for multi-layer launches,
 // whose CTAs wait on one another.
 int layer_tc_max_units(int mode, int pair, bool defer);
-// CUDA-core FP32 layer (k_layer_simt.cu), 128 x 128 tiles.
-cudaError_t launch_layer_simt(const LayerArgs& a, int grid, cudaStream_t s);
+// CUDA-core FP32 layer (k_layer_simt.cu) of the 128 x 128 tile list.
+cudaError_t launch_layer_simt(const LayerArgs& a, cudaStream_t s);
 
 // --- training (k_train.cu) -----------------------------------------------------
 struct ThetaParam {

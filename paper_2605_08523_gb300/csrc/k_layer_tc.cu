@@ -435,17 +435,6 @@ __device__ __forceinline__ void make_lite(const LayerArgs& a, const Tile& t, int
     e.d2 = L.d2;
 }
 
-// Load the 8 state values of row r, columns c0 .. c0 + 7 (two float4 runs 128
-// floats apart in the blocked layout).
-__device__ __forceinline__ void load_state8(const float* S, float* x) {
-    const float4 u = reinterpret_cast<const float4*>(S)[0], w = reinterpret_cast<const float4*>(S + 128)[0];
-    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = w.x; x[5] = w.y; x[6] = w.z; x[7] = w.w;
-}
-__device__ __forceinline__ void store_state8(float* S, const float* x) {
-    reinterpret_cast<float4*>(S)[0] = make_float4(x[0], x[1], x[2], x[3]);
-    reinterpret_cast<float4*>(S + 128)[0] = make_float4(x[4], x[5], x[6], x[7]);
-}
-
 // 256-bit store (sm_100+): dst must be 32-byte aligned.
 __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* w) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]),
@@ -659,16 +648,6 @@ __device__ __forceinline__ void prefetch_tile_state(const LayerArgs& a, const Ti
 
 // ----------------------------------------------------------------------------------
 // OUTFMT: operand format written for the next layer, or kLastLayer.
-// 16-byte asynchronous global -> shared copies through the load/store path
-// (cp.async, L2 only): the store warps' loads do not queue behind the operand
-// tiles in the TMA unit.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // The persistent loop of a unit visits tiles t, t + nunits, ...: is there an
 // active tile after t?  (The last tile of a unit runs its final epilogue inline,
 // so that no store-warp tail follows the last MMAs.)
