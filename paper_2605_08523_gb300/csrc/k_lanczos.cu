@@ -340,113 +340,146 @@ __global__ void __launch_bounds__(kLzSmallThreads, 1) lanczos_small_kernel(Lancz
     }
 }
 
-// number of eigenvalues of the m x m tridiagonal (al, be) below x (Sturm)
-__device__ int sturm_count(const double* al, const double* be, int m, double x) {
+// Number of eigenvalues below x of the m x m tridiagonal with diagonal al and
+// squared off-diagonal b2 (entries of magnitude <= 2): the sign changes of the
+// characteristic polynomials of its leading blocks, p_i = (al_{i-1} - x) p_{i-1}
+// - b2_{i-2} p_{i-2} (Sturm).  A zero counts as a sign change.  No divisions:
+// two dependent FP64 operations a step (a division takes some twenty, and they
+// form one chain).
+__device__ __forceinline__ int sturm_count(const double* al, const double* b2, int m, double x) {
     int cnt = 0;
-    double d = 1.0;
-    for (int i = 0; i < m; ++i) {
-        const double off = i > 0 ? be[i - 1] * be[i - 1] : 0.0;
-        d = (al[i] - x) - (i > 0 ? off / d : 0.0);
-        if (d == 0.0) d = -1e-300;
-        if (d < 0.0) ++cnt;
+    double pp = 1.0, p = al[0] - x;
+    bool neg = !(p > 0.0);                       // sign of p_i, a zero counted opposite to p_{i-1}
+    cnt += neg;
+    for (int i = 1; i < m; ++i) {
+        const double t = fma(al[i] - x, p, -b2[i - 1] * pp);
+        pp = p;
+        p = t;
+        // keep the pair away from underflow (nearly decoupled, nearly equal entries)
+        if (((__double2hiint(p) >> 20) & 0x7ff) < 500 && ((__double2hiint(pp) >> 20) & 0x7ff) < 500) {
+            p *= 0x1p+400;
+            pp *= 0x1p+400;
+        }
+        const bool n2 = p == 0.0 ? !neg : p < 0.0;
+        cnt += n2 != neg;
+        neg = n2;
     }
     return cnt;
 }
 
 // |last entry| of the unit eigenvector for the eigenvalue theta at the edge of
-// the spectrum: inverse iteration with the shift just outside (sign = -1 below
-// the smallest, +1 above the largest), where T - sigma I is definite and the
-// tridiagonal elimination needs no pivoting
-__device__ double edge_vector_last(const double* al, const double* be, int m, double theta, double sign,
-                                   double scale) {
-    double x[kLzSteps], c[kLzSteps], d[kLzSteps];
-    const double sigma = theta + sign * 1e-10 * scale;
-    for (int i = 0; i < m; ++i) x[i] = 1.0;
+// the spectrum: inverse iteration with the shift sigma just outside, where
+// T - sigma I is definite and the tridiagonal elimination needs no pivoting.
+// The factors are formed once (reciprocal pivots), each solve then takes one
+// FMA chain down and one up.
+__device__ __forceinline__ double edge_vector_last(const double* al, const double* be, int m, double sigma) {
+    double x[kLzSteps], r[kLzSteps];             // iterate; 1 / pivot
+#pragma unroll
+    for (int i = 0; i < kLzSteps; ++i) {
+        x[i] = 1.0;
+        r[i] = 0.0;
+        if (i < m) {
+            const double l = i > 0 ? be[i - 1] * r[i > 0 ? i - 1 : 0] : 0.0;
+            r[i] = 1.0 / (i > 0 ? (al[i] - sigma) - l * be[i - 1] : al[i] - sigma);
+        }
+    }
     for (int it = 0; it < 3; ++it) {
-        // solve (T - sigma I) y = x (Thomas algorithm), y into x
-        d[0] = al[0] - sigma;
-        c[0] = x[0];
-        for (int i = 1; i < m; ++i) {
-            const double l = be[i - 1] / d[i - 1];
-            d[i] = (al[i] - sigma) - l * be[i - 1];
-            c[i] = x[i] - l * c[i - 1];
-        }
-        x[m - 1] = c[m - 1] / d[m - 1];
-        for (int i = m - 2; i >= 0; --i) x[i] = (c[i] - be[i] * x[i + 1]) / d[i];
-        double nrm = 0.0;
-        for (int i = 0; i < m; ++i) nrm += x[i] * x[i];
-        nrm = sqrt(nrm);
-        for (int i = 0; i < m; ++i) x[i] /= nrm;
+        // solve (T - sigma I) y = x, y into x
+#pragma unroll
+        for (int i = 1; i < kLzSteps; ++i)
+            if (i < m) x[i] -= (be[i - 1] * r[i - 1]) * x[i - 1];
+        double nrm = 0.0, up = 0.0;              // up = be_i y_{i+1}
+#pragma unroll
+        for (int i = kLzSteps - 1; i >= 0; --i)
+            if (i < m) {
+                x[i] = (x[i] - up) * r[i];
+                nrm += x[i] * x[i];
+                if (i > 0) up = be[i - 1] * x[i];
+            }
+        const double inv = 1.0 / sqrt(nrm);
+#pragma unroll
+        for (int i = 0; i < kLzSteps; ++i) x[i] *= inv;
     }
-    return fabs(x[m - 1]);
+    double last = 0.0;
+#pragma unroll
+    for (int i = 0; i < kLzSteps; ++i)
+        if (i == m - 1) last = fabs(x[i]);
+    return last;
 }
 
-// eigenvalue of T_m at the lower (upper) edge by multisection: the 32 lanes
-// count the eigenvalues below 32 points of the bracket, which shrinks 33-fold
-// per round; 8 rounds leave the edge within 33^-8 < 1e-12 of the bracket (the
-// Gershgorin interval of T), far below the 1 % margin, and inside the 1e-10
-// shift of the residual bound's inverse iteration
-__device__ double edge_eigenvalue(const double* al, const double* be, int m, double lo, double hi, bool upper,
-                                  int lane) {
-    const int target = upper ? m : 1;
-    double l = lo, h = hi;
-    for (int it = 0; it < 8; ++it) {
-        const double x = l + (h - l) * (double)(lane + 1) / 33.0;
-        const bool hit = sturm_count(al, be, m, x) >= target;
-        const unsigned mask = __ballot_sync(0xffffffffu, hit);
-        if (mask == 0u) {
-            l = __shfl_sync(0xffffffffu, x, 31);
-        } else {
-            const int k = __ffs(mask) - 1;
-            const double xk = __shfl_sync(0xffffffffu, x, k);
-            const double xk1 = __shfl_sync(0xffffffffu, x, k > 0 ? k - 1 : 0);
-            if (k > 0) l = xk1;
-            h = xk;
-        }
-    }
-    return h;
-}
-
-// one warp per instance
-__global__ void lanczos_bounds_kernel(LanczosArgs a) {
-    __shared__ double sal[4][kLzSteps], sbe[4][kLzSteps];
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const int b = blockIdx.x * 4 + wi;
-    if (b >= a.nb) return;
+// Two warps per instance: warp 0 the lower edge of the spectrum of T_m, warp 1
+// the upper one.  The edge eigenvalue by multisection: the 32 lanes count the
+// eigenvalues below 32 points of the bracket, which shrinks 33-fold per round;
+// 8 rounds leave the edge within 33^-8 < 1e-12 of the bracket (the Gershgorin
+// interval of T), far below the 1 % margin, and inside the 1e-10 shift of the
+// residual bound's inverse iteration.  Bound by the latency of dependent FP64
+// operations; one instance took 379 us with one warp, divisions in the Sturm
+// counts and the factors formed anew in each solve, 84 us now.
+__global__ void __launch_bounds__(64) lanczos_bounds_kernel(LanczosArgs a) {
+    __shared__ double al[kLzSteps], be[kLzSteps], sal[kLzSteps], sb2[kLzSteps];
+    __shared__ double edge[2], res[2];
+    const int lane = threadIdx.x & 31, upper = threadIdx.x >> 5;
+    const int b = blockIdx.x;
     const int m = a.state[b] & (kLzStopped - 1);
     if (m < 1) return;
     const double* ab = a.ab + (size_t)b * kLzSteps * 2;
-    double* al = sal[wi];
-    double* be = sbe[wi];
-    for (int i = lane; i < m; i += 32) {
-        al[i] = ab[2 * i];
-        be[i] = ab[2 * i + 1];
+    if (threadIdx.x < m) {
+        al[threadIdx.x] = ab[2 * threadIdx.x];
+        be[threadIdx.x] = ab[2 * threadIdx.x + 1];
     }
-    __syncwarp();
+    __syncthreads();
+    // Gershgorin interval of T (lane i: row i)
+    double lo = 1e300, hi = -1e300;
     bool finite = true;
-    double lo = 1e300, hi = -1e300;             // Gershgorin interval of T
-    for (int i = 0; i < m; ++i) {
-        finite = finite && isfinite(al[i]) && isfinite(be[i]);
-        const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < m ? fabs(be[i]) : 0.0);
-        lo = fmin(lo, al[i] - r);
-        hi = fmax(hi, al[i] + r);
+    if (lane < m) {
+        finite = isfinite(al[lane]) && isfinite(be[lane]);
+        const double r = (lane > 0 ? fabs(be[lane - 1]) : 0.0) + (lane + 1 < m ? fabs(be[lane]) : 0.0);
+        lo = al[lane] - r;
+        hi = al[lane] + r;
     }
-    if (!finite) return;                         // the Gershgorin bounds stay (and flag the input)
-    const double tmin = edge_eigenvalue(al, be, m, lo, hi, false, lane);
-    const double tmax = edge_eigenvalue(al, be, m, lo, hi, true, lane);
-    if (lane != 0) return;
+    if (!__all_sync(0xffffffffu, finite)) return;   // the Gershgorin bounds stay (and flag the input)
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    // in units of the interval, from its lower end: T' = (T - lo) 2^-e
+    const int ex = hi > lo ? ilogb(hi - lo) : 0;
+    if (threadIdx.x < m) {
+        const double f = scalbn(be[threadIdx.x], -ex);
+        sal[threadIdx.x] = scalbn(al[threadIdx.x] - lo, -ex);
+        sb2[threadIdx.x] = f * f;
+    }
+    __syncthreads();
+    double l = 0.0, h = scalbn(hi - lo, -ex);
+    const int target = upper ? m : 1;
+    if (h > 0.0)
+        for (int it = 0; it < 8; ++it) {
+            const double x = l + (h - l) * ((double)(lane + 1) * (1.0 / 33.0));
+            const bool hit = sturm_count(sal, sb2, m, x) >= target;
+            const unsigned mask = __ballot_sync(0xffffffffu, hit);
+            const int k = mask ? __ffs(mask) - 1 : 32;       // the first point with enough eigenvalues below
+            const double xk = __shfl_sync(0xffffffffu, x, k & 31);
+            const double xk1 = __shfl_sync(0xffffffffu, x, k > 0 ? k - 1 : 0);
+            if (k > 0) l = xk1;
+            if (k < 32) h = xk;
+        }
+    if (lane == 0) edge[upper] = lo + scalbn(h, ex);
+    __syncthreads();
+    const double tmin = edge[0], tmax = edge[1];
     const double scale = fmax(fabs(tmin), fabs(tmax)) + (tmax - tmin) + 1e-300;
-    double rmin = 0.0, rmax = 0.0;
-    const double blast = be[m - 1];
-    if (m > 1 && blast > 0.0) {
-        rmin = blast * edge_vector_last(al, be, m, tmin, -1.0, scale);
-        rmax = blast * edge_vector_last(al, be, m, tmax, +1.0, scale);
-    } else if (m == 1) {
-        rmin = rmax = blast;
+    if (lane == 0) {
+        const double blast = be[m - 1];
+        double r = 0.0;
+        if (m > 1 && blast > 0.0)
+            r = blast * edge_vector_last(al, be, m, upper ? tmax + 1e-10 * scale : tmin - 1e-10 * scale);
+        else if (m == 1) r = blast;
+        res[upper] = r;
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     // 1 % of the Ritz spread, plus 1e-6 of the Ritz magnitude for the FP32 products
     const double delta = 0.01 * (tmax - tmin) + 1e-6 * fmax(fabs(tmin), fabs(tmax));
-    const double elo = tmin - rmin - delta, ehi = tmax + rmax + delta;
+    const double elo = tmin - res[0] - delta, ehi = tmax + res[1] + delta;
     const double glo = dunkey(a.iw[b].kmin), ghi = dunkey(a.iw[b].kmax);
     if (!(isfinite(elo) && isfinite(ehi) && isfinite(glo) && isfinite(ghi))) return;
     // intersected with the Gershgorin interval, each end kept inside it
@@ -494,7 +527,7 @@ void launch_lanczos(const LanczosArgs& a, int max_n, int sms, cudaStream_t s) {
         }
         lanczos_queue_kernel<<<(a.nb + 255) / 256, 256, 0, s>>>(a);
         lanczos_small_kernel<<<std::min(a.nb, std::max(1, sms)), kLzSmallThreads, kLzSmallCacheBytes, s>>>(a);
-        lanczos_bounds_kernel<<<(a.nb + 3) / 4, 128, 0, s>>>(a);
+        lanczos_bounds_kernel<<<a.nb, 64, 0, s>>>(a);
         count_launch(3);
         return;
     }
@@ -507,7 +540,7 @@ void launch_lanczos(const LanczosArgs& a, int max_n, int sms, cudaStream_t s) {
         lanczos_update_kernel<<<a.nb, kLzThreads, 0, s>>>(a, j);
         count_launch(2);
     }
-    lanczos_bounds_kernel<<<(a.nb + 3) / 4, 128, 0, s>>>(a);
+    lanczos_bounds_kernel<<<a.nb, 64, 0, s>>>(a);
     count_launch();
 }
 
