@@ -81,8 +81,10 @@ typedef enum {
 #define FTSP2_REFINE2       0x8  /* last two layers in FTSP2_FP32 arithmetic  */
 /* Tile shape of the tensor-core layer launches.  By default a batch runs with
  * the shape ftsp2_autotune recorded for it or, if none was recorded, with the
- * shape a padding model prefers; these two flags override both. */
-#define FTSP2_PAIR_TILES    0x10 /* 256 x 256 tiles on CTA pairs (cta_group::2) */
+ * shape a model of the layer's time prefers; these two flags override both. */
+#define FTSP2_PAIR_TILES    0x10 /* tiles on CTA pairs (cta_group::2): 256 rows by
+                                    256 or 128 columns, whichever the model of
+                                    the layer's time prefers                  */
 #define FTSP2_SINGLE_TILES  0x20 /* 128 x 128 tiles on single CTAs             */
 /* Spectral bounds: by default the Gershgorin interval of Appendix A.  With this
  * flag it is tightened by 24 Lanczos steps in FP64 (start vector from
@@ -380,7 +382,7 @@ ftsp2_status ftsp2_density_mu(const double* dH, const ftsp2_instance* inst, ftsp
  * that call; the results of the last run are left in them).  For each shape
  * the batch runs once untimed and then `reps` times between CUDA events on
  * `stream`; ms[0] receives the mean time of the 128 x 128 single-CTA shape,
- * ms[1] that of the 256 x 256 pair shape (ms nullable), *choice the shape kept
+ * ms[1] that of the pair shape (ms nullable), *choice the shape kept
  * (0 single, 1 pair; -1 in FTSP2_FP32 mode, which has no tensor-core layers and
  * is not timed).  The record is keyed by device, mode, density/entropy
  * selection, refinement flags and the sorted list of orders n, lives for the
@@ -398,7 +400,7 @@ ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst,
 /* The tile shape a call with these arguments would use on the current device:
  * 1 pair, 0 single, -1 none (FTSP2_FP32 mode).  `want` as in
  * ftsp2_workspace_size.  *from_tuner is set to 1 if the shape comes from an
- * ftsp2_autotune record, 0 if from the flags or the padding model.  Host-only
+ * ftsp2_autotune record, 0 if from the flags or the time model.  Host-only
  * apart from reading the device's SM count. */
 ftsp2_status ftsp2_tile_shape(const ftsp2_instance* inst, int nb, ftsp2_mode mode, int want,
                               int flags, int* shape, int* from_tuner);

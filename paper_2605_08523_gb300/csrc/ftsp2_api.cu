@@ -74,7 +74,8 @@ static PFN_cuTensorMapEncodeTiled_v12000 encoder() {
 }
 
 // 2-D map over a stack of nb padded P x P slabs (rows = nb * P), element type
-// `dt`, box {box_k elements, box_rows rows}, 128-byte swizzle.
+// `dt`, box {box_k elements, box_rows rows} of 128-byte (64-byte) rows with the
+// 128-byte (64-byte) swizzle.
 static bool encode_map(CUtensorMap* m, void* base, CUtensorMapDataType dt, int esize, int P, int nb, int box_k,
                        int box_rows) {
     auto fn = encoder();
@@ -84,7 +85,8 @@ static bool encode_map(CUtensorMap* m, void* base, CUtensorMapDataType dt, int e
     cuuint32_t box[2] = {(cuuint32_t)box_k, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, dt, 2, base, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    box_k * esize == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -430,15 +432,28 @@ static int chunk_elems_of(int mode, int g, int Lmax, double mean_k) {
 static int refine_layers(int flags) { return (flags & FTSP2_REFINE2) ? 2 : ((flags & FTSP2_REFINE1) ? 1 : 0); }
 
 static int host_tiles_of(int n, int BM, int BN) {
-    const int q = BN / BM;
     const int nI = (n + BM - 1) / BM;
     const int nJ = (n + BN - 1) / BN;
     int c = 0;
-    for (int J = 0; J < nJ; ++J) c += std::min(q * (J + 1), nI);
+    for (int J = 0; J < nJ; ++J) c += std::min(((J + 1) * BN + BM - 1) / BM, nI);
     return c;
 }
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+// Deferred final epilogue of the 256 x 256 tiles: by default when their mean K is
+// long enough for two store warps to keep up with the MMAs.
+static bool deferred_epilogue(const ftsp2_instance* inst, int nb, int flags) {
+    if (flags & FTSP2_EPI_INLINE) return false;
+    if (flags & FTSP2_EPI_DEFERRED) return true;
+    double tile_k = 0.0, tiles = 0.0;          // sum of the orders n over the tiles; tiles
+    for (int b = 0; b < nb; ++b) {
+        const double t = (double)host_tiles_of(inst[b].n, tc_block_m(SHAPE_PAIR), tc_block_n(SHAPE_PAIR));
+        tiles += t;
+        tile_k += t * inst[b].n;
+    }
+    return tile_k >= (double)kDeferMinK * tiles;
+}
 
 static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want, int flags, Layout& L,
                          int planes = 2) {
@@ -453,35 +468,24 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     const int P = (int)align_up((size_t)maxn, kPad);
     const int nch = want == 3 ? 2 : 1;
     const bool simt_main = mode == FTSP2_FP32;
-    // main tile table: 256 x 256 pair tiles (tensor-core modes) or 128 x 128
-    // (FP32 mode); the 128 x 128 table serves single-CTA tensor-core layers and
-    // FP32 refinement layers
-    const int BN = simt_main ? 128 : tc_block_n(mode, 1);
-    const int BM = simt_main ? 128 : tc_block_m(mode, 1);
     const bool refine = !simt_main && refine_layers(flags) > 0;
-    const bool need_ref = !simt_main;
-    long long nt = 0, ntr = 0;
-    double tile_k = 0.0;                       // sum of the orders n over the pair tiles
-    for (int b = 0; b < nb; ++b) {
-        const long long t = host_tiles_of(inst[b].n, BM, BN);
-        nt += t;
-        tile_k += (double)t * inst[b].n;
-        if (need_ref) ntr += host_tiles_of(inst[b].n, 128, 128);
+    // tiles of each shape; the tile of a call's main table is that of its shape
+    // (128 x 128 in FP32 mode), a second table of 128 x 128 tiles serves
+    // single-CTA layers and FP32 refinement layers
+    long long nt[3] = {0, 0, 0};
+    for (int b = 0; b < nb; ++b)
+        for (int sh = 0; sh < 3; ++sh) nt[sh] += host_tiles_of(inst[b].n, tc_block_m(sh), tc_block_n(sh));
+    const bool defer = !simt_main && deferred_epilogue(inst, nb, flags);
+    long long ntmax = 0;
+    for (int sh = 0; sh < 3; ++sh) {
+        nt[sh] *= nch;
+        ntmax = std::max(ntmax, nt[sh]);
     }
-    // deferred final epilogue of the pair tiles: by default when their mean
-    // K is long enough for two store warps to keep up with the MMAs
-    const bool defer = !simt_main && !(flags & FTSP2_EPI_INLINE) &&
-                       ((flags & FTSP2_EPI_DEFERRED) || tile_k >= (double)kDeferMinK * (double)nt);
-    nt *= nch;
-    ntr *= nch;
-    if (nt > (1ll << 30)) return FTSP2_E_ARG;
+    if (ntmax > (1ll << 30)) return FTSP2_E_ARG;
     L.P = P;
     L.nb = nb;
     L.nchains = nch;
-    L.ntiles = (int)nt;
-    L.ntiles_ref = (int)ntr;
-    L.BN = BN;
-    L.BM = BM;
+    for (int sh = 0; sh < 3; ++sh) L.ntiles[sh] = (int)nt[sh];
     L.plane_elems = (size_t)nb * P * P;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -492,11 +496,11 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     L.status = take(256);
     L.done = take(sizeof(int) * kMaxLayers * kMaxChains * (size_t)nb);
     L.inst_work = take(sizeof(InstWork) * nb);
-    L.tiles = take(sizeof(Tile) * nt);
-    L.tiles_ref = need_ref ? take(sizeof(Tile) * ntr) : 0;
-    L.partials = take(sizeof(double) * 2 * kPartialSlots * std::max<long long>(nt, ntr));
+    L.tiles = take(sizeof(Tile) * ntmax);
+    L.tiles_ref = simt_main ? 0 : take(sizeof(Tile) * nt[SHAPE_SINGLE]);
+    L.partials = take(sizeof(double) * 2 * kPartialSlots * ntmax);
     L.lanczos = take(lanczos_ws_bytes(nb, P));   // used with FTSP2_LANCZOS only
-    L.escr_ctas = defer ? (int)std::min<long long>(kMaxDeferCtas, 2 * nt) : 0;
+    L.escr_ctas = defer ? (int)std::min<long long>(kMaxDeferCtas, 2 * nt[SHAPE_PAIR]) : 0;
     L.escr = L.escr_ctas ? take((size_t)L.escr_ctas * kEpiScratchFloats * sizeof(float)) : 0;
     const int fmt = fmt_of_mode(mode);
     for (int c = 0; c < kMaxChains; ++c) {
@@ -525,11 +529,12 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
 
 static ftsp2_status from_cuda(cudaError_t e) { return e == cudaSuccess ? FTSP2_OK : FTSP2_E_CUDA; }
 
-// ---- tile-shape choice (autotuner) --------------------------------------------
-// Tensor-core layers run either on CTA pairs with 256 x 256 tiles or on single
-// CTAs with 128 x 128 tiles.  The choice is per batch signature (device, mode,
-// chains, refinement, the sorted list of orders n): ftsp2_autotune measures both
-// and records the faster; otherwise a padding model decides.
+// ---- tile-shape choice --------------------------------------------------------
+// Tensor-core layers run on single CTAs with 128 x 128 tiles or on CTA pairs with
+// 256 x 256 or 256 x 128 tiles.  Single or pair is forced by a flag, or recorded
+// by ftsp2_autotune per batch signature (device, mode, chains, refinement, the
+// sorted list of orders n); otherwise, and for the width of the pair tiles, the
+// cost model below decides.
 static std::mutex g_tune_mu;
 static std::map<uint64_t, int> g_tune;
 
@@ -553,9 +558,12 @@ static uint64_t batch_signature(const ftsp2_instance* inst, int nb, int mode, in
     return h;
 }
 
-// Padding model: multiply-adds issued per layer (tiles x tile^2 x n) divided by
-// the number of units that run them in parallel, with the waves rounded up.
-static int shape_by_model(const ftsp2_instance* inst, int nb, int sms) {
+// Accumulation chunks (below) are set by the mean order over the tiles of the
+// shape that this padding model prefers: multiply-adds issued per layer (tiles x
+// tile^2 x n) over the units that run them in parallel, in whole waves.  It is
+// part of what a solve computes, so it stays as it is while the launches' own
+// shape follows the measured costs.
+static int chunk_shape(const ftsp2_instance* inst, int nb, int sms) {
     double cost[2] = {0.0, 0.0};
     for (int pair = 0; pair < 2; ++pair) {
         const int T = pair ? 256 : 128;
@@ -569,26 +577,72 @@ static int shape_by_model(const ftsp2_instance* inst, int nb, int sms) {
         }
         const double waves = std::ceil((double)tiles / std::max(1, units));
         const double per_tile = work / std::max<long long>(1, tiles);
-        // a pair tile moves half of B per SM; count its MMA work at 0.8
         cost[pair] = waves * per_tile / (pair ? 2.0 : 1.0) * (pair ? 0.8 : 1.0);
     }
     return cost[1] <= cost[0] ? 1 : 0;
 }
 
-static int tile_shape_choice(const ftsp2_instance* inst, int nb, int mode, int want, int flags, int sms,
-                             int* from_tuner = nullptr) {
+// Clocks of one layer with a tile shape, from the measured parts of a tile: the
+// K loop per 64 elements (the MMAs of a pair: 768 clocks of FP16X2 on 128
+// columns run in 850, on 256 columns 1536 in 1570; a single CTA's 128 x 128
+// MMAs, both panels from one shared memory, take 1430 for 768), and the final
+// epilogue, which follows the K loop when a unit has one tile and otherwise
+// overlaps the next tile's (kStream is then its share of a tile, bound by the
+// state's traffic).  With more tiles than units the layer costs its mean load,
+// and a part of a tile for the uneven end: less when other instances or chains
+// fill it.  Measured (one lattice, density + entropy, FP16X2; single / 256 x 256 /
+// 256 x 128, us per solve): n = 64: 214 / 287 / 223; 256: 275 / 587 / 266;
+// 1024: 508 / 846 / 429; 2048: 1367 / 1324 / 1130; 3072: 4013 / 3946 / 3192;
+// 4096: 9175 / 7388 / 7731; 40 instances of n = 256: 985 / 1325 / 1095;
+// the ragged batch of 512: 22980 / 34750 / 25170.
+static double shape_cost(const ftsp2_instance* inst, int nb, int nch, int mode, int sms, int shape, bool deferred) {
+    static const double kSlice[3][3] = {{2860, 3140, 1700}, {2500, 3100, 1650}, {1430, 1570, 850}};   // TF32X3, BF16X3, FP16X2
+    const double slice = kSlice[mode == FTSP2_TF32X3 ? 0 : mode == FTSP2_BF16X3 ? 1 : 2][shape];
+    const double epi = shape == SHAPE_SINGLE ? 7000 : shape == SHAPE_PAIR128 ? 7700 : 28000;
+    const double stream = shape == SHAPE_PAIR && !deferred ? 28000 : 14000;
+    const double units = std::max(1, shape == SHAPE_SINGLE ? sms : sms / 2);
+    double tiles = 0.0, load = 0.0, longest = 0.0;
+    for (int b = 0; b < nb; ++b) {
+        const double t = (double)nch * (double)host_tiles_of(inst[b].n, tc_block_m(shape), tc_block_n(shape));
+        const double k = slice * std::ceil(inst[b].n / 64.0);
+        tiles += t;
+        load += t * std::max(k, stream);
+        longest = std::max(longest, k);
+    }
+    if (tiles <= units) return longest + epi;
+    return load / units + (nb * nch == 1 ? 0.5 : 0.35) * load / tiles;
+}
+
+// The forced or recorded choice of a call: 1 pair, 0 single, -1 neither.
+static int chosen_pair(const ftsp2_instance* inst, int nb, int mode, int want, int flags, int* from_tuner = nullptr) {
     if (from_tuner) *from_tuner = 0;
     if (flags & FTSP2_PAIR_TILES) return 1;
     if (flags & FTSP2_SINGLE_TILES) return 0;
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune.find(batch_signature(inst, nb, mode, want, flags));
-        if (it != g_tune.end()) {
-            if (from_tuner) *from_tuner = 1;
-            return it->second;
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    auto it = g_tune.find(batch_signature(inst, nb, mode, want, flags));
+    if (it == g_tune.end()) return -1;
+    if (from_tuner) *from_tuner = 1;
+    return it->second;
+}
+
+// Shape of a call's tensor-core layers: the cheapest by the model within the
+// forced or recorded choice (pair < 0: none).  Pair tiles forced together with a
+// placement of their final epilogue are the 256 x 256 ones, which have the choice.
+static int layer_shape(const ftsp2_instance* inst, int nb, int mode, int want, int flags, int pair, int sms,
+                       bool deferred) {
+    if ((flags & FTSP2_PAIR_TILES) && (flags & (FTSP2_EPI_DEFERRED | FTSP2_EPI_INLINE))) return SHAPE_PAIR;
+    const int nch = want == 3 ? 2 : 1;
+    int best = -1;
+    double cost = 0.0;
+    for (int shape = 0; shape < 3; ++shape) {
+        if (pair >= 0 && pair != (shape != SHAPE_SINGLE)) continue;
+        const double c = shape_cost(inst, nb, nch, mode, sms, shape, deferred);
+        if (best < 0 || c < cost) {
+            best = shape;
+            cost = c;
         }
     }
-    return shape_by_model(inst, nb, sms);
+    return best;
 }
 
 // The launch sequence of (a1)-(a6).
@@ -639,7 +693,12 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     int* dstatus = reinterpret_cast<int*>(W + L.status);
     InstWork* iw = reinterpret_cast<InstWork*>(W + L.inst_work);
     Tile* tiles = reinterpret_cast<Tile*>(W + L.tiles);
-    Tile* tiles_ref = L.ntiles_ref ? reinterpret_cast<Tile*>(W + L.tiles_ref) : nullptr;
+    // tile shape of the tensor-core layers; the second table (128 x 128) only
+    // serves FP32 refinement layers beside larger tiles
+    const int pair_choice = all_simt ? 0 : chosen_pair(inst, nb, mode, want, flags);
+    const int shape = all_simt ? SHAPE_SINGLE
+                               : layer_shape(inst, nb, mode, want, flags, pair_choice, di.sms, L.escr_ctas > 0);
+    Tile* tiles_ref = (shape != SHAPE_SINGLE && R > 0 && !refine_tc) ? reinterpret_cast<Tile*>(W + L.tiles_ref) : nullptr;
     double* partials = reinterpret_cast<double*>(W + L.partials);
 
     SetupArgs sa;
@@ -649,10 +708,8 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     sa.P = L.P;
     sa.Lmax = Lmax;
     sa.nchains = L.nchains;
-    sa.BN = L.BN;
-    sa.BM = L.BM;
-    sa.BN_ref = 128;
-    sa.BM_ref = 128;
+    sa.BM = tc_block_m(shape);
+    sa.BN = tc_block_n(shape);
     sa.models = models;
     sa.nmodels = (int)set->host.size();
     sa.flags = flags;
@@ -705,39 +762,35 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     }
     launch_init(ia, maxn, s);
 
-    // tensor maps of both parities (tensor-core layers only)
-    TmaMaps maps[2];
-    if (!all_simt && refine_from > 0) {
-        const CUtensorMapDataType dt = fmt == OP_F16X2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                       : fmt == OP_BF16X3 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                                          : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-        const int es = fmt == OP_TF32X3 ? 4 : 2;
-        const int nsplit = fmt == OP_BF16X3 ? 3 : 2;
-        const int bke = 128 / es;
-        std::memset(maps, 0, sizeof(maps));
+    // tensor maps of the operand planes of both parities, read and written (main
+    // format; refinement layers)
+    TmaMaps maps[2], mapsR[2];
+    WriteMaps wmaps[2], wmapsR[2];
+    auto encode = [&](TmaMaps* rd, WriteMaps* wr, const size_t (&op)[kMaxChains][2], int fm) {
+        const CUtensorMapDataType dt = fm == OP_F16X2    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                       : fm == OP_BF16X3 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                         : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+        const int es = (fm == OP_F16X2 || fm == OP_BF16X3) ? 2 : 4;
+        const int nsplit = op_bytes(fm) / es;
         for (int p = 0; p < 2; ++p)
             for (int c = 0; c < L.nchains; ++c)
                 for (int sp = 0; sp < nsplit; ++sp) {
-                    void* base = W + L.OP[c][p] + (size_t)sp * es * L.plane_elems;
-                    if (!encode_map(&maps[p].a[c][sp], base, dt, es, L.P, nb, bke, kTileM)) return FTSP2_E_CUDA;
-                    // transposed 64 x 64 panels of the upper triangle (16-bit planes)
-                    if (es == 2 && !encode_map(&maps[p].t[c][sp], base, dt, es, L.P, nb, 64, 64))
-                        return FTSP2_E_CUDA;
+                    void* base = W + op[c][p] + (size_t)sp * es * L.plane_elems;
+                    if (rd && !encode_map(&rd[p].a[c][sp], base, dt, es, L.P, nb, 128 / es, kTileM)) return false;
+                    if (rd && !encode_map(&rd[p].t[c][sp], base, dt, es, L.P, nb, 128 / es, 64)) return false;
+                    if (!encode_map(&wr[p].w[c][sp], base, dt, es, L.P, nb, 64 / es, 32)) return false;
                 }
+        return true;
+    };
+    if (!all_simt && refine_from > 0) {
+        std::memset(maps, 0, sizeof(maps));
+        std::memset(wmaps, 0, sizeof(wmaps));
+        if (!encode(maps, wmaps, L.OP, fmt)) return FTSP2_E_CUDA;
     }
-    // tensor maps of the BF16X3 refinement operands (FTSP2_REFINE_TC)
-    TmaMaps mapsR[2];
-    if (refine_tc && R > 0) {
+    if (R > 0) {
         std::memset(mapsR, 0, sizeof(mapsR));
-        for (int p = 0; p < 2; ++p)
-            for (int c = 0; c < L.nchains; ++c)
-                for (int sp = 0; sp < 3; ++sp) {
-                    void* base = W + L.OPR[c][p] + (size_t)sp * 2 * L.plane_elems;
-                    if (!encode_map(&mapsR[p].a[c][sp], base, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L.P, nb, 64, kTileM))
-                        return FTSP2_E_CUDA;
-                    if (!encode_map(&mapsR[p].t[c][sp], base, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, L.P, nb, 64, 64))
-                        return FTSP2_E_CUDA;
-                }
+        std::memset(wmapsR, 0, sizeof(wmapsR));
+        if (!encode(refine_tc ? mapsR : nullptr, wmapsR, L.OPR, rfmt)) return FTSP2_E_CUDA;
     }
 
     LayerArgs la;
@@ -764,12 +817,12 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     }
     auto is_simt = [&](int g) { return all_simt || (g >= refine_from && !refine_tc); };
     auto is_rtc = [&](int g) { return refine_tc && g >= refine_from; };
-    const int pair = all_simt ? 1 : tile_shape_choice(inst, nb, mode, want, flags, di.sms);
-    // mean order n over the tensor-core tiles of the chosen shape (chunk policy)
+    const bool pair = shape != SHAPE_SINGLE;
+    // mean order n over the tiles that set the accumulation chunks
     double mean_k = 0.0;
     {
         double wk = 0.0, wt = 0.0;
-        const int T = pair ? 256 : 128;
+        const int T = (pair_choice >= 0 ? pair_choice : chunk_shape(inst, nb, di.sms)) ? 256 : 128;
         for (int b = 0; b < nb; ++b) {
             const double t = (double)host_tiles_of(inst[b].n, T, T);
             wt += t;
@@ -821,23 +874,20 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
             else la.opr[c] = W + L.OP[c][rp];
             if (next_simt || next_rtc) la.opw[c] = all_simt ? W + L.OP[c][wp] : W + L.OPR[c][wp];
             else la.opw[c] = W + L.OP[c][wp];
-            // write operands of layer g + 1 (same kind): parity (g + 2) & 1
-            la.opw_alt[c] = (rtc ? W + L.OPR[c][rp] : W + L.OP[c][rp]);
         }
         if (dD == nullptr && la.last) la.D = nullptr;
         cudaError_t e;
         if (simt) {
-            const bool use_ref = !all_simt;
-            la.tiles = use_ref ? tiles_ref : tiles;
-            la.ntiles = use_ref ? L.ntiles_ref : L.ntiles;
+            la.tiles = tiles_ref ? tiles_ref : tiles;
+            la.ntiles = L.ntiles[SHAPE_SINGLE];
             e = launch_layer_simt(la, s);
-            last_table = use_ref ? 1 : 0;
+            last_table = tiles_ref ? 1 : 0;
         } else {
-            la.tiles = pair ? tiles : tiles_ref;
-            la.ntiles = pair ? L.ntiles : L.ntiles_ref;
-            la.dtab = pair ? 0 : 1;
+            la.tiles = tiles;
+            la.ntiles = L.ntiles[shape];
+            la.dtab = 0;
             const int units = std::max(1, std::min(la.ntiles, pair ? di.sms / 2 : di.sms));
-            la.escr = pair && L.escr_ctas >= 2 * units ? reinterpret_cast<float*>(W + L.escr) : nullptr;
+            la.escr = shape == SHAPE_PAIR && L.escr_ctas >= 2 * units ? reinterpret_cast<float*>(W + L.escr) : nullptr;
             // consecutive layers of this kind in one persistent launch when each
             // layer is only a few waves of tiles (at most 8), and every unit can
             // be resident at once (the launch's CTAs wait on one another).  With
@@ -854,14 +904,15 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
                 while (g + m < Lmax && in_run(g + m)) ++m;
                 if (m > 1) {
                     // at most the co-resident units (cluster placement may leave an SM out)
-                    const bool defer = pair && la.escr != nullptr;
-                    const int maxu = layer_tc_max_units(lmode, pair, defer);
+                    const int maxu = layer_tc_max_units(lmode, shape, la.escr != nullptr);
                     if (maxu >= units) lunits = units;
                     else if (maxu >= (units * 9) / 10) lunits = maxu;
                     else m = 1;
                 }
             }
             la.nlayers = m;
+            // one tile per unit: its state stays on the chip between the layers
+            la.resident = m > 1 && la.ntiles == lunits ? 1 : 0;
             if (m > 1) {
                 // chunk schedule over the run: chunk_elems up to tail_from, chunk_tail after
                 for (int h = g + 1; h < g + m; ++h) {
@@ -882,17 +933,21 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
                     e0 = e1 = nullptr;
                 }
             }
-            const TmaMaps& m0 = rtc ? mapsR[g & 1] : maps[g & 1];
-            const TmaMaps& m1 = rtc ? mapsR[(g + 1) & 1] : maps[(g + 1) & 1];
-            e = launch_layer_tc(lmode, la, m0, m1, m > 1 ? lunits : units, pair, s);
+            // read and written by this layer, and by the next one of the launch
+            const int rp = g & 1, wp = rp ^ 1;
+            const TmaMaps* const rd = rtc ? mapsR : maps;
+            const WriteMaps* const wr = (next_rtc || next_simt) ? wmapsR : wmaps;
+            const LayerMaps lm = {{&rd[rp], &rd[wp]}, {&wr[wp], &wr[rp]}};
+            e = launch_layer_tc(lmode, la, lm, m > 1 ? lunits : units, shape, s);
             if (m > 1) {
                 if (e != cudaSuccess && !capturing) {
                     // multi-layer launches refused here: one launch per layer from now on
                     cudaGetLastError();
                     g_coop_ok.store(0);
                     la.nlayers = m = 1;
+                    la.resident = 0;
                     la.tail_from = INT_MAX;
-                    e = launch_layer_tc(lmode, la, m0, m1, units, pair, s);
+                    e = launch_layer_tc(lmode, la, lm, units, shape, s);
                 } else if (e == cudaSuccess) {
                     g_coop_ok.store(1);
                 }
@@ -902,7 +957,7 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
                 std::lock_guard<std::mutex> lk(g_prof_mu);
                 g_prof_events.push_back(ProfEvent{e0, e1, m});
             }
-            last_table = pair ? 0 : 1;
+            last_table = 0;
             g += m - 1;     // the run's remaining layers are done
         }
         if (e != cudaSuccess) return FTSP2_E_CUDA;
@@ -1224,6 +1279,7 @@ ftsp2_status ftsp2_rescale(const double* dH, const ftsp2_instance* inst, const f
     sa.iw = reinterpret_cast<InstWork*>(W + 1024);
     sa.tiles = nullptr;
     sa.tiles_ref = nullptr;
+    sa.BM = sa.BN = 128;
     sa.rec = dRec;
     sa.status = reinterpret_cast<int*>(W);
     sa.h32 = (flags & FTSP2_LANCZOS) ? reinterpret_cast<float*>(W + h32_off) : nullptr;
@@ -1378,7 +1434,8 @@ ftsp2_status ftsp2_tile_shape(const ftsp2_instance* inst, int nb, ftsp2_mode mod
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return FTSP2_E_CUDA;
-    *shape = tile_shape_choice(inst, nb, mode, want, flags, sms, from_tuner);
+    const int pair = chosen_pair(inst, nb, mode, want, flags, from_tuner);
+    *shape = layer_shape(inst, nb, mode, want, flags, pair, sms, deferred_epilogue(inst, nb, flags)) != SHAPE_SINGLE;
     return FTSP2_OK;
 }
 

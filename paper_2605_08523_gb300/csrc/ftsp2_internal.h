@@ -30,7 +30,7 @@ int max_nparams(int L);                      // L (L + 5) / 2 + 2 numbers of a f
 constexpr int kMaxChains = 2;
 constexpr int kTileM = 128;                  // tensor-core tile rows (UMMA M)
 constexpr int kPad = 128;                    // matrix pitch granularity (elements)
-constexpr int kPartialSlots = 32;            // FP64 partial-sum slots per tile (last layer)
+constexpr int kPartialSlots = 16;            // FP64 partial-sum slots per tile (last layer)
 constexpr int kEpiScratchFloats = 32768;     // deferred epilogue: finished sums of one CTA's tile
 constexpr int kMaxDeferCtas = 192;           // CTAs with a scratch slot in the workspace
 constexpr int kDeferMinK = 3072;             // default: deferred epilogue from this mean tile K
@@ -101,6 +101,12 @@ struct InstWork {
     int tile_count[2][kMaxChains];
     int start_layer;                 // per chain, 16 bits each: first global layer
     int nonfinite;
+    // what the layer launches need of an instance (decide kernel)
+    int n, active;                   // order; the instance has a valid model
+    int layer_off[kMaxChains];       // first DevLayer of each chain's table
+    int flip;
+    float cdiag;                     // added on the diagonal of D: f0, or 1 - f0 when flipped
+    long long doff;                  // element offset of D
 };
 
 struct Layout {
@@ -112,7 +118,8 @@ struct Layout {
     size_t Z[kMaxChains], A[kMaxChains], OP[kMaxChains][2], OPR[kMaxChains][2];
     size_t total;
     size_t plane_elems;   // nb * P * P
-    int P, nb, nchains, ntiles, ntiles_ref, BN, BM;
+    int P, nb, nchains;
+    int ntiles[3];        // tiles of each shape over all chains: 128 x 128, 256 x 256, 256 x 128
     int planes;           // FP32 state planes per chain: 2 (Z, A), or L + 1 for Max-SP2 tables
 };
 
@@ -120,7 +127,7 @@ struct Layout {
 struct SetupArgs {
     const double* H;
     const ftsp2_instance* inst;
-    int nb, P, Lmax, nchains, BM, BN, BM_ref, BN_ref;
+    int nb, P, Lmax, nchains, BM, BN;  // tile of the main table (the second one: 128 x 128)
     const DevModel* models;
     int nmodels;
     int flags;
@@ -225,7 +232,7 @@ struct LayerArgs {
     float* Z[kMaxChains];             // state (blocked layout); A[c] == Z[c] + plane_elems
     float* A[kMaxChains];
     const uint8_t* opr[kMaxChains];   // read operands (plane 0 base) - SIMT path
-    uint8_t* opw[kMaxChains];         // write operands (plane 0 base)
+    uint8_t* opw[kMaxChains];         // write operands (plane 0 base) - SIMT path
     size_t plane_elems;
     float* D;
     double* partials;
@@ -240,14 +247,11 @@ struct LayerArgs {
     // Several consecutive layers in one persistent launch (nlayers > 1): the
     // work items are (global layer gl + l, tile) for l < nlayers, taken in that
     // order; an item of layer g waits until every epilogue of layer g - 1 of its
-    // chain has finished (done[(g - 1) * kMaxChains + chain] reaches
-    // kEpiWarps x CTAs per tile x tiles per chain).  Layers gl + 1, gl + 3, ...
-    // write their operands through opw_alt and read them through the second
-    // tensor-map set.  Layers >= tail_from accumulate chunk_tail elements per
-    // TMEM chunk instead of chunk_elems.
+    // instance and chain has finished.  Layers gl + 1, gl + 3, ... read and write
+    // their operands through the second tensor-map sets.  Layers >= tail_from
+    // accumulate chunk_tail elements per TMEM chunk instead of chunk_elems.
     int nlayers;
     int chunk_tail, tail_from;
-    uint8_t* opw_alt[kMaxChains];
     // completion counters of multi-layer launches, one per (layer, instance,
     // chain): done_inst[(g * nb + instance) * kMaxChains + chain]; an item waits
     // for its own instance's previous layer
@@ -264,25 +268,39 @@ struct LayerArgs {
     // one completion more than their predecessor layer can give, so that the
     // dependency wait runs out; -1 in normal operation.
     int stall_layer;
+    // Every unit has one and the same tile in all layers of the launch: the
+    // state of that tile stays in TMEM between them (128-column tiles).
+    int resident;
 };
 
 struct TmaMaps {
     CUtensorMap a[kMaxChains][3];   // [chain][split plane], boxes of 128 rows x 128 bytes
-    CUtensorMap t[kMaxChains][3];   // 16-bit planes: boxes of 64 rows x 64 columns (transposed panels)
+    // boxes of 64 rows x 128 bytes: B panels of 64 rows, and (16-bit planes) the
+    // 64 x 64 halves of transposed panels
+    CUtensorMap t[kMaxChains][3];
 };
 
-// Tensor-core layer (k_layer_tc.cu); mode in {TF32X3, BF16X3, FP16X2}.
-int tc_block_n(int mode, int pair);
-int tc_block_m(int mode, int pair);
-int tc_smem_bytes(int mode);
-// pair = 1: 256 x 256 tiles on CTA pairs (units = pairs); pair = 0: 128 x 128
-// tiles on single CTAs (units = CTAs).  Persistent grid of `units`.
-cudaError_t launch_layer_tc(int mode, const LayerArgs& a, const TmaMaps& maps, const TmaMaps& maps_alt, int units,
-                            int pair, cudaStream_t s);
+// Boxes of 32 rows x 64 bytes (64-byte swizzle) of the operand planes a layer writes.
+struct WriteMaps {
+    CUtensorMap w[kMaxChains][3];
+};
+// The maps of a launch: operands read and written by its even and odd layers.
+struct LayerMaps {
+    const TmaMaps* rd[2];
+    const WriteMaps* wr[2];
+};
+
+// Tensor-core layer (k_layer_tc.cu); mode in {TF32X3, BF16X3, FP16X2}; shape 0:
+// 128 x 128 tiles on single CTAs (units = CTAs), 1: 256 x 256 and 2: 256 x 128
+// tiles on CTA pairs (units = pairs).  Persistent grid of `units`.
+enum { SHAPE_SINGLE = 0, SHAPE_PAIR = 1, SHAPE_PAIR128 = 2 };
+int tc_block_m(int shape);
+int tc_block_n(int shape);
+cudaError_t launch_layer_tc(int mode, const LayerArgs& a, const LayerMaps& m, int units, int shape, cudaStream_t s);
 // Largest number of units (pairs or CTAs) of the main-format layer kernel that
 // can be resident at once (0 if unknown): the bound for multi-layer launches,
 // whose CTAs wait on one another.
-int layer_tc_max_units(int mode, int pair, bool defer);
+int layer_tc_max_units(int mode, int shape, bool defer);
 // CUDA-core FP32 layer (k_layer_simt.cu) of the 128 x 128 tile list.
 cudaError_t launch_layer_simt(const LayerArgs& a, cudaStream_t s);
 

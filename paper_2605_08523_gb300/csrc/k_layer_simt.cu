@@ -37,7 +37,7 @@ constexpr int kSThreads = 128;
 constexpr int kSWarps = kSThreads / 32;
 constexpr int kSPitch = kSQ + 1; // pitch of the staged sums
 static_assert(kSStages * 2 * kSK * kSQ >= kSQ * kSPitch, "the ring holds the staged sums");
-static_assert(4 * kSWarps <= kPartialSlots, "one partial-sum slot per warp and quadrant");
+static_assert(4 * kSWarps == kPartialSlots, "one partial-sum slot per warp and quadrant");
 
 typedef unsigned long long f32x2;      // two packed FP32 values
 
@@ -59,10 +59,8 @@ __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_c
     const int n = a.inst[tl.inst].n;
     const int rowA = tl.I * 128 + (quad >> 1) * kSQ, rowB = tl.J * 128 + (quad & 1) * kSQ;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // this quadrant's slots of the tile's FP64 partial sums, and the slots no warp has
+    // this warp's slot of the tile's FP64 partial sums
     const size_t slot = (size_t)t * kPartialSlots + quad * kSWarps + warp;
-    if (a.last && quad == 0 && tid < 2 * (kPartialSlots - 4 * kSWarps))
-        a.partials[((size_t)t * kPartialSlots + 4 * kSWarps) * 2 + tid] = 0.0;
     if (rowA > rowB || rowA >= n || rowB >= n) {
         if (a.last && lane < 2) a.partials[slot * 2 + lane] = 0.0;
         return;

@@ -17,17 +17,20 @@ namespace ftsp2 {
 
 // ------------------------------------------------------------------------------
 // prep: one block.  Initialises the bound keys and writes the tile tables.
-// Tile (I, J) of an instance covers rows [128 I, 128 I + 128) and columns
+// Tile (I, J) of an instance covers rows [BM I, BM I + BM) and columns
 // [BN J, BN J + BN); only tiles touching the upper triangle are listed
-// (I < q (J + 1), q = BN / 128).  Chain-major order: all tiles of chain 0, then
+// (BM I < BN (J + 1)).  Chain-major order: all tiles of chain 0, then
 // chain 1; inside a chain, instance by instance.
 // ------------------------------------------------------------------------------
+// rows of tiles in tile column J
+__device__ __forceinline__ int tiles_in_column(int J, int nI, int BM, int BN) {
+    return min(((J + 1) * BN + BM - 1) / BM, nI);
+}
 __device__ __forceinline__ int tiles_of(int n, int BM, int BN) {
-    const int q = BN / BM;
     const int nI = (n + BM - 1) / BM;
     const int nJ = (n + BN - 1) / BN;
     int c = 0;
-    for (int J = 0; J < nJ; ++J) c += min(q * (J + 1), nI);
+    for (int J = 0; J < nJ; ++J) c += tiles_in_column(J, nI, BM, BN);
     return c;
 }
 
@@ -108,7 +111,6 @@ __device__ void block_exclusive_scan_fill(const ftsp2_instance* inst, int nb, in
         }
     }
     __syncthreads();
-    const int q = BN / BM;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T >> 5;
     for (int b = warp; b < nb; b += nw) {
         const int n = inst[b].n;
@@ -117,7 +119,7 @@ __device__ void block_exclusive_scan_fill(const ftsp2_instance* inst, int nb, in
         for (int l = lane; l < cnt; l += 32) {
             int J = 0, rem = l;
             for (;;) {
-                const int col = min(q * (J + 1), nI);
+                const int col = tiles_in_column(J, nI, BM, BN);
                 if (rem < col) break;
                 rem -= col;
                 ++J;
@@ -144,7 +146,7 @@ __global__ void prep_kernel(SetupArgs a) {
         for (int i = threadIdx.x; i < cnt; i += blockDim.x) a.done[i] = 0;
     }
     if (a.tiles) block_exclusive_scan_fill(a.inst, a.nb, a.BM, a.BN, a.nchains, a.iw, a.tiles, 0);
-    if (a.tiles_ref) block_exclusive_scan_fill(a.inst, a.nb, a.BM_ref, a.BN_ref, a.nchains, a.iw, a.tiles_ref, 1);
+    if (a.tiles_ref) block_exclusive_scan_fill(a.inst, a.nb, 128, 128, a.nchains, a.iw, a.tiles_ref, 1);
 }
 
 void launch_prep(const SetupArgs& a, cudaStream_t s) {
@@ -336,8 +338,16 @@ __global__ void decide_kernel(SetupArgs a) {
         }
     }
     a.rec[b] = r;
-    a.iw[b].start_layer = sl[0] | (sl[1] << 16);
-    if (r.status == FTSP2_OK && r.model >= 0) {
+    InstWork& w = a.iw[b];
+    w.start_layer = sl[0] | (sl[1] << 16);
+    w.n = in.n;
+    w.active = r.status == FTSP2_OK && r.model >= 0;
+    w.flip = r.flip;
+    w.doff = in.offset;
+    if (w.active) {
+        const DevModel& M = a.models[r.model];
+        for (int c = 0; c < a.nchains; ++c) w.layer_off[c] = a.chain_kind[c] == CHAIN_ENTROPY ? M.offS : M.off;
+        w.cdiag = (float)(r.flip ? 1.0 - M.f0 : M.f0);
         int first = sl[0];
         for (int c = 1; c < a.nchains; ++c) first = min(first, sl[c]);
         atomicMin(&a.status[1], first);
