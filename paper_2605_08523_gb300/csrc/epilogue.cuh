@@ -40,6 +40,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+__device__ __forceinline__ void store_partial(const LayerArgs& a, int inst, int chain, int rb, int cb, double tr,
+                                              double sq) {
+    double2* const p = reinterpret_cast<double2*>(a.partials) +
+                       ((size_t)inst * a.nchains + chain) * partial_blocks(a.P) + partial_index(rb, cb);
+    *p = make_double2(tr, sq);
+}
+
 struct EpiCtx {
     int n, P, chain, kind, flip, last, next_fmt;
     float mul;            // multiplier of the product: a_k, times 2^(-2 e_k) for scaled FP16 operands

@@ -498,7 +498,7 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     L.inst_work = take(sizeof(InstWork) * nb);
     L.tiles = take(sizeof(Tile) * ntmax);
     L.tiles_ref = simt_main ? 0 : take(sizeof(Tile) * nt[SHAPE_SINGLE]);
-    L.partials = take(sizeof(double) * 2 * kPartialSlots * ntmax);
+    L.partials = take(sizeof(double) * 2 * (size_t)nb * nch * partial_blocks(P));
     L.lanczos = take(lanczos_ws_bytes(nb, P));   // used with FTSP2_LANCZOS only
     L.escr_ctas = defer ? (int)std::min<long long>(kMaxDeferCtas, 2 * nt[SHAPE_PAIR]) : 0;
     L.escr = L.escr_ctas ? take((size_t)L.escr_ctas * kEpiScratchFloats * sizeof(float)) : 0;
@@ -830,7 +830,6 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
         }
         mean_k = wt > 0.0 ? wk / wt : 0.0;
     }
-    int last_table = 0;
     // Operands of 16-bit tensor-core layers are stored as the upper triangle
     // plus the diagonal tile blocks when the layer that reads them can load the
     // rest transposed (FP16X2, BF16X3); the mirror is written everywhere before
@@ -845,7 +844,10 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     auto in_run = [&](int h) {
         return h < Lmax - 1 && !is_simt(h) && !is_simt(h + 1) && is_rtc(h) == is_rtc(h + 1);
     };
-    for (int g = 0; g < Lmax; ++g) {
+    const int max_units = pair ? di.sms / 2 : di.sms;
+    la.done_inst = reinterpret_cast<int*>(W + L.done);
+    la.nb = nb;
+    for (int g = 0; g < Lmax;) {
         const bool simt = is_simt(g);
         const bool next_simt = g + 1 < Lmax && is_simt(g + 1);
         const bool rtc = is_rtc(g);
@@ -866,8 +868,6 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
         la.mirror_all = (next_tc16 && !(flags & FTSP2_FULL_OPERANDS)) ? 0 : 1;
         la.lower_t = (!simt && prev_skips_mirror) ? 1 : 0;
         prev_skips_mirror = la.mirror_all ? 0 : 1;
-        la.done_inst = reinterpret_cast<int*>(W + L.done);
-        la.nb = nb;
         for (int c = 0; c < L.nchains; ++c) {
             const int rp = g & 1, wp = (g + 1) & 1;
             if (simt || rtc) la.opr[c] = all_simt ? W + L.OP[c][rp] : W + L.OPR[c][rp];
@@ -875,29 +875,28 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
             if (next_simt || next_rtc) la.opw[c] = all_simt ? W + L.OP[c][wp] : W + L.OPR[c][wp];
             else la.opw[c] = W + L.OP[c][wp];
         }
-        if (dD == nullptr && la.last) la.D = nullptr;
         cudaError_t e;
+        int m = 1;                             // layers of this launch
         if (simt) {
             la.tiles = tiles_ref ? tiles_ref : tiles;
             la.ntiles = L.ntiles[SHAPE_SINGLE];
             e = launch_layer_simt(la, s);
-            last_table = tiles_ref ? 1 : 0;
         } else {
             la.tiles = tiles;
             la.ntiles = L.ntiles[shape];
             la.dtab = 0;
-            const int units = std::max(1, std::min(la.ntiles, pair ? di.sms / 2 : di.sms));
+            const int units = std::max(1, std::min(la.ntiles, max_units));
             la.escr = shape == SHAPE_PAIR && L.escr_ctas >= 2 * units ? reinterpret_cast<float*>(W + L.escr) : nullptr;
             // consecutive layers of this kind in one persistent launch when each
-            // layer is only a few waves of tiles (at most 8), and every unit can
-            // be resident at once (the launch's CTAs wait on one another).  With
-            // more waves the idle tail of a launch is a small share, and runs
-            // measured slower: at n = 8192 the busier GPU ran at a lower
-            // power-capped clock (90.2 against 83.2 ms per solve), and on the
-            // 512-instance ragged batch (71 waves) the units drifted apart
-            // without a barrier per layer, the instances in flight at once
-            // outgrew the L2, and the batch took 34.2 against 31.0 ms.
-            int m = 1, lunits = units;
+            // layer is only a few waves of tiles, and every unit can be resident at
+            // once (the launch's CTAs wait on one another).  With more waves the
+            // idle tail of a launch is a small share, and runs measured slower: at
+            // n = 8192 the busier GPU ran at a lower power-capped clock (90.2
+            // against 83.2 ms per solve, an earlier kernel).  The ragged batch of
+            // 512 in runs over groups of instances whose working sets stay in the
+            // L2 (48, 80, 120 MB) took 27.4, 25.7 and 25.0 ms against 23.1: a tile
+            // is bound by its own latency, not by HBM.
+            int lunits = units;
             if (!(flags & FTSP2_LAYER_LAUNCHES) && g_coop_ok.load() != 0 && !(capturing && g_coop_ok.load() != 1) &&
                 la.ntiles <= 8 * units && in_run(g) &&
                 (lmode == FTSP2_TF32X3 || la.lower_t == (la.mirror_all ? 0 : 1))) {
@@ -957,10 +956,9 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
                 std::lock_guard<std::mutex> lk(g_prof_mu);
                 g_prof_events.push_back(ProfEvent{e0, e1, m});
             }
-            last_table = 0;
-            g += m - 1;     // the run's remaining layers are done
         }
         if (e != cudaSuccess) return FTSP2_E_CUDA;
+        g += m;
     }
     FinalArgs fa;
     fa.inst = dInst;
@@ -968,7 +966,7 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     fa.models = models;
     fa.iw = iw;
     fa.partials = partials;
-    fa.table = last_table;
+    fa.P = L.P;
     fa.nb = nb;
     fa.nchains = L.nchains;
     fa.chain_kind[0] = kinds[0];

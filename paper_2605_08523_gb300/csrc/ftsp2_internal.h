@@ -30,7 +30,6 @@ int max_nparams(int L);                      // L (L + 5) / 2 + 2 numbers of a f
 constexpr int kMaxChains = 2;
 constexpr int kTileM = 128;                  // tensor-core tile rows (UMMA M)
 constexpr int kPad = 128;                    // matrix pitch granularity (elements)
-constexpr int kPartialSlots = 16;            // FP64 partial-sum slots per tile (last layer)
 constexpr int kEpiScratchFloats = 32768;     // deferred epilogue: finished sums of one CTA's tile
 constexpr int kMaxDeferCtas = 192;           // CTAs with a scratch slot in the workspace
 constexpr int kDeferMinK = 3072;             // default: deferred epilogue from this mean tile K
@@ -162,6 +161,7 @@ struct InitArgs {
     int refine_fmt;                // OP_F32 (CUDA-core refinement) or OP_BF16X3 (FTSP2_REFINE_TC)
     int refine_from;               // global layers >= refine_from are refinement layers on OPR
     int upper_only;                // 16-bit operands as the upper triangle plus diagonal blocks
+    int cols;                      // columns per CTA (launch_init)
     size_t plane_elems;
 };
 void launch_init(const InitArgs& a, int max_n, cudaStream_t s);
@@ -171,9 +171,8 @@ struct FinalArgs {
     ftsp2_rescale_rec* rec;
     const DevModel* models;
     const InstWork* iw;
-    const double* partials;   // [tile][kPartialSlots][2]
-    int table;                // tile table used by the last layer (0 main, 1 128x128)
-    int nb, nchains;
+    const double* partials;   // partial_blocks(P) pairs per instance and chain
+    int nb, nchains, P;
     int chain_kind[kMaxChains];
     double* trace;            // nullable, [nb][2]
     double* S;                // nullable, [nb]
@@ -339,6 +338,15 @@ void train_sample_grid(double beta0, double mu0, int N, uint64_t seed, double* x
 void train_init_mlsp2(int L, double beta0, double mu0, double* theta);
 void train_init_alt(int L, double mu0, double* alt);
 void mlsp2_to_skip(int L, const double* theta, double* tab);
+
+// FP64 partial sums of the last layer: a pair (sum of the diagonal, sum of the
+// squares) per 32 x 64 block (row block rb, column block cb) of the upper triangle
+// (rb <= 2 cb + 1), by position, whatever the tiles that computed it.
+__host__ __device__ __forceinline__ int partial_index(int rb, int cb) { return cb * (cb + 1) + rb; }
+__host__ __device__ __forceinline__ int partial_blocks(int n) {
+    const int B = (n + 63) / 64;
+    return (B - 1) * B + ((n + 31) / 32 < 2 * B ? (n + 31) / 32 : 2 * B);
+}
 
 // Element offset of (r, c) inside one P x P slab of the FP32 state Z, A (P a
 // multiple of 128).  The slab is cut into blocks of 32 rows x 8 columns (1 KB),

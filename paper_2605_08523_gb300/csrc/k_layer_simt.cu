@@ -37,7 +37,6 @@ constexpr int kSThreads = 128;
 constexpr int kSWarps = kSThreads / 32;
 constexpr int kSPitch = kSQ + 1; // pitch of the staged sums
 static_assert(kSStages * 2 * kSK * kSQ >= kSQ * kSPitch, "the ring holds the staged sums");
-static_assert(4 * kSWarps == kPartialSlots, "one partial-sum slot per warp and quadrant");
 
 typedef unsigned long long f32x2;      // two packed FP32 values
 
@@ -59,12 +58,7 @@ __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_c
     const int n = a.inst[tl.inst].n;
     const int rowA = tl.I * 128 + (quad >> 1) * kSQ, rowB = tl.J * 128 + (quad & 1) * kSQ;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // this warp's slot of the tile's FP64 partial sums
-    const size_t slot = (size_t)t * kPartialSlots + quad * kSWarps + warp;
-    if (rowA > rowB || rowA >= n || rowB >= n) {
-        if (a.last && lane < 2) a.partials[slot * 2 + lane] = 0.0;
-        return;
-    }
+    if (rowA > rowB || rowA >= n || rowB >= n) return;
     const float* const Op = reinterpret_cast<const float*>(a.opr[tl.chain]) + (size_t)tl.inst * a.P * a.P;
     // outputs of a thread: rows 8 ty .. + 7, columns 4 tx .. + 3 (a warp covers 32 x 32)
     const int ty = (warp >> 1) * 4 + (lane >> 3), tx = (warp & 1) * 8 + (lane & 7);
@@ -157,14 +151,20 @@ __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_c
         else epi_segment(a, e, r, c0, v, tr, sq);
     }
     if (a.last) {
+        // warps w and w + 2 have the column groups of one 32 x 64 block
+        __shared__ double red[kSWarps][2];
         for (int o = 16; o > 0; o >>= 1) {
             tr += __shfl_xor_sync(0xffffffffu, tr, o);
             sq += __shfl_xor_sync(0xffffffffu, sq, o);
         }
         if (lane == 0) {
-            a.partials[slot * 2 + 0] = tr;
-            a.partials[slot * 2 + 1] = sq;
+            red[warp][0] = tr;
+            red[warp][1] = sq;
         }
+        __syncthreads();
+        if (tid < 2 && rowA + 32 * tid < n)
+            store_partial(a, tl.inst, tl.chain, (rowA >> 5) + tid, rowB >> 6, red[tid][0] + red[tid + 2][0],
+                          red[tid][1] + red[tid + 2][1]);
     }
 }
 

@@ -153,7 +153,6 @@ static_assert(kDeferWarps * kItemFloats == kEpiScratchFloats, "scratch of one CT
 // to the kDeferWarps that the accumulating warps give for an inline tile
 static_assert(kDeferWarps % kStoreWarps == 0, "completion shares of the store warps");
 constexpr int kDeferThreads = 64 + 32 * (kDeferWarps + kStoreWarps);
-static_assert(kPartialSlots == 2 * kEpiWarps, "one partial-sum slot per epilogue warp of the pair");
 
 // split planes (s, t) of the products Z_s Z_t, in issue order
 __host__ __device__ constexpr int prod_a(int p) { return p == 2 ? 1 : (p == 4 ? 2 : (p == 5 ? 1 : 0)); }
@@ -553,7 +552,7 @@ struct __align__(16) ItemCtx {
     int n, nk, ck;            // order, K slices, K slices per accumulation chunk (nk = 0: end of the list)
     int row0, col0;           // first row of the CTA's block, first column of the tile
     int mirror;               // operands (c, r) are written too
-    int t;                    // tile index (partial sums)
+    int inst;                 // instance
     // TMA producer
     int slab_row;             // first row of the instance's slab in the operand maps
     int chain, maps;          // chain; tensor-map set
@@ -826,58 +825,64 @@ __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c
 // unit of this GPU.  The direct row (r, c .. c + 7) is written as two 16-byte
 // vectors when the whole group lies in the triangle and is aligned; the mirror
 // (c, r) is one element per lane, a contiguous run of row c across the warp.
+struct LastSums {
+    double tr, sq;
+    float lo;
+};
 __device__ __forceinline__ void epi_last32(const LayerArgs& a, const ItemCtx& c, int R0, int lane, int c0,
-                                           const float (&v)[32], State32& s, int c_next, double& tr, double& sq,
-                                           float& lo) {
+                                           const float (&v)[32], const State32& s, LastSums& b) {
     const int n = c.n, r = R0 + lane;
     const float mul = c.mul, bp = c.bp, d = c.d, g1 = c.g, cdiag = c.cdiag;
     const bool flip = c.flip != 0, dout = c.dout != 0;
     float* const Db = a.D + c.doff;
     float* const drow = Db + (int64_t)r * n;
+    if (r >= n) return;
+    double tr = b.tr, sq = b.sq;
+    float lo = b.lo;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
         const int cc0 = c0 + 8 * h;
-        if (cc0 < n && r < n) {
-            float dv[8];
-            float sh = 0.f, sl = 0.f;
+        if (cc0 >= n) break;
+        float dv[8];
+        float sh = 0.f, sl = 0.f;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int cc = cc0 + u;
-                const float z = s.z[h >> 1][8 * (h & 1) + u], x = s.x[h >> 1][8 * (h & 1) + u];
-                const float g = fmaf(g1, fmaf(mul, v[8 * h + u], bp * z), fmaf(d, z, x));
-                const bool diag = r == cc;
-                if (flip) dv[u] = (diag ? cdiag : 0.f) - g;
-                else dv[u] = g + (diag ? cdiag : 0.f);
-                if (cc < n && r <= cc) {
-                    if (diag) tr += (double)g;
-                    const float w = diag ? g : 2.f * g;            // (r, c) and (c, r)
-                    const float p = __fmul_rn(w, g);
-                    const float pe = fmaf(w, g, -p);               // w g - p, exact
-                    const float t = __fadd_rn(sh, p);
-                    const float bb = __fsub_rn(t, sh);
-                    const float te = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), __fsub_rn(p, bb));   // sh + p - t, exact
-                    sh = t;
-                    sl = __fadd_rn(sl, __fadd_rn(te, pe));
-                }
-            }
-            sq += (double)sh;
-            lo = __fadd_rn(lo, sl);
-            if (dout) {
-                if (cc0 >= r && cc0 + 8 <= n && (reinterpret_cast<uintptr_t>(drow + cc0) & 15u) == 0) {
-                    reinterpret_cast<float4*>(drow + cc0)[0] = make_float4(dv[0], dv[1], dv[2], dv[3]);
-                    reinterpret_cast<float4*>(drow + cc0)[1] = make_float4(dv[4], dv[5], dv[6], dv[7]);
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (cc0 + u < n && r <= cc0 + u) drow[cc0 + u] = dv[u];
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (cc0 + u < n && r < cc0 + u) Db[(int64_t)(cc0 + u) * n + r] = dv[u];
+        for (int u = 0; u < 8; ++u) {
+            const int cc = cc0 + u;
+            const float z = s.z[h >> 1][8 * (h & 1) + u], x = s.x[h >> 1][8 * (h & 1) + u];
+            const float g = fmaf(g1, fmaf(mul, v[8 * h + u], bp * z), fmaf(d, z, x));
+            const bool diag = r == cc;
+            if (flip) dv[u] = (diag ? cdiag : 0.f) - g;
+            else dv[u] = g + (diag ? cdiag : 0.f);
+            if (cc < n && r <= cc) {
+                if (diag) tr += (double)g;
+                const float w = diag ? g : 2.f * g;            // (r, c) and (c, r)
+                const float p = __fmul_rn(w, g);
+                const float pe = fmaf(w, g, -p);               // w g - p, exact
+                const float t = __fadd_rn(sh, p);
+                const float bb = __fsub_rn(t, sh);
+                const float te = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), __fsub_rn(p, bb));   // sh + p - t, exact
+                sh = t;
+                sl = __fadd_rn(sl, __fadd_rn(te, pe));
             }
         }
-        if ((h & 1) && c_next >= 0) load16(a, c.Z, n, R0, r, c_next + 8 * (h - 1), s.z[h >> 1], s.x[h >> 1]);
+        sq += (double)sh;
+        lo = __fadd_rn(lo, sl);
+        if (!dout) continue;
+        if (cc0 >= r && cc0 + 8 <= n && (reinterpret_cast<uintptr_t>(drow + cc0) & 15u) == 0) {
+            reinterpret_cast<float4*>(drow + cc0)[0] = make_float4(dv[0], dv[1], dv[2], dv[3]);
+            reinterpret_cast<float4*>(drow + cc0)[1] = make_float4(dv[4], dv[5], dv[6], dv[7]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (cc0 + u < n && r <= cc0 + u) drow[cc0 + u] = dv[u];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (cc0 + u < n && r < cc0 + u) Db[(int64_t)(cc0 + u) * n + r] = dv[u];
     }
+    b.tr = tr;
+    b.sq = sq;
+    b.lo = lo;
 }
 
 // L2 prefetch of the Z and A state that the CTA's epilogue warps read at the
@@ -940,10 +945,10 @@ __device__ __forceinline__ bool next_block(const ItemCtx& c, int sw, int& e) {
     }
 }
 
-// What the final epilogue of tile t (tl) needs: instance w, layer constants L.
+// What the final epilogue of tile tl needs: instance w, layer constants L.
 template <int MODE, int OUTFMT, int SHAPE>
 __device__ __forceinline__ void fill_epilogue(const LayerArgs& a, const Tile& tl, const InstWork& w, const DevLayer& L,
-                                              int t, int rank, ItemCtx& c) {
+                                              int rank, ItemCtx& c) {
     using G = Geo<SHAPE>;
     c.Z = a.Z[tl.chain] + (size_t)tl.inst * a.P * a.P;
     c.os = OUTFMT == OP_F16X2 ? L.out_scale : 1.f;
@@ -963,7 +968,7 @@ __device__ __forceinline__ void fill_epilogue(const LayerArgs& a, const Tile& tl
     c.row0 = tl.I * G::TM + rank * kCtaRows;
     c.col0 = tl.J * G::TN;
     c.mirror = a.mirror_all || (tl.J * G::TN) / G::TM == tl.I;   // inside the diagonal block, or everywhere
-    c.t = t;
+    c.inst = tl.inst;
     c.slab_row = tl.inst * a.P;
 }
 
@@ -1054,62 +1059,62 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t tmem = tmem_slot;
 
     if (warp == kCtxWarp) {
-        if (lane == 0) {
-            // ---------------- context warp: the unit's active items ----------------
-            const int nf = a.ntiles * a.nlayers;
-            // the items of layers before the first active one are left out
-            const int f0 = max(0, first_layer - a.gl) * a.ntiles;
-            int it = 0, pt = -1;
-            bool ok = true;
+        // ---------------- context warp: the unit's active items ----------------
+        // 32 items are looked up at a time, a lane each (a model with few layers
+        // starts late: many items of a ragged batch are inactive).
+        const int nf = a.ntiles * a.nlayers;
+        // the items of layers before the first active one are left out
+        const int f0 = max(0, first_layer - a.gl) * a.ntiles + unit;
+        int it = 0;
+        bool ok = true;
+        for (int fb = f0; fb < nf && ok; fb += 32 * nunits) {
+            const int f = fb + lane * nunits;
+            const int l = f / a.ntiles, g = a.gl + l, t = f - l * a.ntiles;
             Tile tl = {0, 0, 0, 0};
-            const InstWork* w = nullptr;
-            int start = 0, active = 0;
-            for (int f = f0 + unit; f < nf && ok; f += nunits) {
-                const int l = f / a.ntiles, g = a.gl + l, t = f - l * a.ntiles;
-                if (t != pt) {
-                    tl = a.tiles[t];
-                    w = a.iw + tl.inst;
-                    start = (w->start_layer >> (16 * tl.chain)) & 0xffff;
-                    active = w->active;
-                    pt = t;
+            int k = -1;
+            if (f < nf) {
+                tl = a.tiles[t];
+                const InstWork& w = a.iw[tl.inst];
+                if (w.active) k = g - ((w.start_layer >> (16 * tl.chain)) & 0xffff);
+            }
+            unsigned active = __ballot_sync(0xffffffffu, k >= 0);
+            for (; active && ok; active &= active - 1) {
+                if (lane == __ffs(active) - 1) {
+                    const InstWork& w = a.iw[tl.inst];
+                    const DevLayer L = a.layers[w.layer_off[tl.chain] + k];
+                    const int slot = it % kCtxSlots;
+                    ok = wait_bar(&ctx_empty[slot], ((it / kCtxSlots) & 1) ^ 1u, a);
+                    if (ok) {
+                        ItemCtx& c = ctx[slot];
+                        const int odd = l & 1;
+                        fill_epilogue<MODE, OUTFMT, SHAPE>(a, tl, w, L, (int)rank, c);
+                        const int n = c.n;
+                        c.nk = (n + BKE - 1) / BKE;
+                        const int ce = g >= a.tail_from ? a.chunk_tail : a.chunk_elems;
+                        c.ck = max(1, (ce > 0 ? ce : C::CK * BKE) / BKE);
+                        const int blkB = (tl.J * TN) / TM;             // diagonal block of the B panel
+                        c.chain = tl.chain;
+                        c.maps = odd;
+                        c.panA = c.row0;
+                        c.panB = c.col0 + (int)rank * G::BROWS;
+                        c.lowA = (!C::TF32 && a.lower_t) ? tl.I * TM / BKE : 0;
+                        c.lowB = (!C::TF32 && a.lower_t) ? blkB * TM / BKE : 0;
+                        c.same = SHAPE == SHAPE_SINGLE && tl.I == tl.J;
+                        // operands and state written by other CTAs of this launch
+                        const bool dep = g > a.gl && k > 0;
+                        c.dep = dep ? inst_counter(a, g - 1, tl.inst, tl.chain) : nullptr;
+                        c.target = kEpiWarps * G::NCTA * w.tile_count[a.dtab][tl.chain] + (g == a.stall_layer ? 1 : 0);
+                        c.done = inst_counter(a, g, tl.inst, tl.chain);
+                        c.first = it == 0;
+                        c.final = l == a.nlayers - 1;
+                        mbar_arrive(&ctx_full[slot]);
+                    }
                 }
-                const int k = g - start;
-                if (!active || k < 0) {
-                    // an inactive item counts as finished for the layer's completion
-                    if (a.nlayers > 1) atomicAdd(inst_counter(a, g, tl.inst, tl.chain), kEpiWarps);
-                    continue;
-                }
-                const DevLayer L = a.layers[w->layer_off[tl.chain] + k];
-                const int slot = it % kCtxSlots;
-                if (!wait_bar(&ctx_empty[slot], ((it / kCtxSlots) & 1) ^ 1u, a)) {
-                    ok = false;
-                    break;
-                }
-                ItemCtx& c = ctx[slot];
-                const int odd = (g - a.gl) & 1;
-                fill_epilogue<MODE, OUTFMT, SHAPE>(a, tl, *w, L, t, (int)rank, c);
-                const int n = c.n;
-                c.nk = (n + BKE - 1) / BKE;
-                const int ce = g >= a.tail_from ? a.chunk_tail : a.chunk_elems;
-                c.ck = max(1, (ce > 0 ? ce : C::CK * BKE) / BKE);
-                const int blkB = (tl.J * TN) / TM;             // diagonal block of the B panel
-                c.chain = tl.chain;
-                c.maps = odd;
-                c.panA = c.row0;
-                c.panB = c.col0 + (int)rank * G::BROWS;
-                c.lowA = (!C::TF32 && a.lower_t) ? tl.I * TM / BKE : 0;
-                c.lowB = (!C::TF32 && a.lower_t) ? blkB * TM / BKE : 0;
-                c.same = SHAPE == SHAPE_SINGLE && tl.I == tl.J;
-                // operands and state written by other CTAs of this launch
-                const bool dep = g > a.gl && g - 1 >= first_layer;
-                c.dep = dep ? inst_counter(a, g - 1, tl.inst, tl.chain) : nullptr;
-                c.target = kEpiWarps * G::NCTA * w->tile_count[a.dtab][tl.chain] + (g == a.stall_layer ? 1 : 0);
-                c.done = inst_counter(a, g, tl.inst, tl.chain);
-                c.first = it == 0;
-                c.final = g == a.gl + a.nlayers - 1;
-                mbar_arrive(&ctx_full[slot]);
+                ok = __all_sync(0xffffffffu, ok);
                 ++it;
             }
+        }
+        if (lane == 0) {
             const int slot = it % kCtxSlots;
             if (ok && wait_bar(&ctx_empty[slot], ((it / kCtxSlots) & 1) ^ 1u, a)) {
                 ctx[slot].nk = 0;                    // the end of the list
@@ -1426,18 +1431,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (!ok) break;
             // skip mode (warp-uniform): the protocol without the memory work
             const bool work = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&abort_flag) == 0 ? 1 : 0, 0) != 0;
-            double tr = 0.0, sq = 0.0;
-            if (live && work) {
-                const CUtensorMap* const wm = (c.maps ? wmaps1 : wmaps0).w[c.chain];
-                const bool from_tmem = resident && !c.first, to_tmem = resident && !c.final;
-                float lo = 0.f;
-                auto block = [&](int cb, float (&v)[32], State32& s) {
-                    const int next = cb + 32 < cb1 ? C0 + cb + 32 : -1;
-                    if constexpr (LAST) epi_last32(a, c, R0, lane, C0 + cb, v, s, next, tr, sq, lo);
-                    else
-                        epi_block32<OUTFMT, CAN_RESIDE>(a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem,
-                                                        to_tmem, v, s, next);
-                };
+            const bool from_tmem = CAN_RESIDE && resident && !c.first, to_tmem = CAN_RESIDE && resident && !c.final;
+            // every block of the warp: its sums in v, the state loaded ahead in s
+            auto blocks = [&](auto&& block) {
                 if constexpr (HOLD) {
                     State32 s;
                     load_first(s);
@@ -1455,8 +1451,45 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     if (cb0 == 0) block(0, v0, ahead);
                     if (cb1 == EPI_COLS) block(EPI_COLS - 32, v1, ahead);
                 }
-                if constexpr (LAST) sq += (double)lo;
-                if (CAN_RESIDE && to_tmem) tmem_wait_st();
+            };
+            auto next_of = [&](int cb) { return cb + 32 < cb1 ? C0 + cb + 32 : -1; };
+            if constexpr (!LAST) {
+                if (live && work) {
+                    const CUtensorMap* const wm = (c.maps ? wmaps1 : wmaps0).w[c.chain];
+                    blocks([&](int cb, float (&v)[32], State32& s) {
+                        epi_block32<OUTFMT, CAN_RESIDE>(a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem,
+                                                        to_tmem, v, s, next_of(cb));
+                    });
+                    if (CAN_RESIDE && to_tmem) tmem_wait_st();
+                }
+            }
+            if constexpr (LAST) {
+                // the sums of every 32 x 64 block of the matrix apart (the same
+                // ones whatever the tiles), in the order of their position
+                LastSums lb;
+                lb.tr = lb.sq = 0.0;
+                lb.lo = 0.f;
+                auto flush = [&](int col) {
+                    double tr = lb.tr, sq = lb.sq + (double)lb.lo;
+                    for (int o = 16; o > 0; o >>= 1) {
+                        tr += __shfl_xor_sync(0xffffffffu, tr, o);
+                        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                    }
+                    if (lane == 0) store_partial(a, c.inst, c.chain, R0 >> 5, col >> 6, tr, sq);
+                    lb.tr = lb.sq = 0.0;
+                    lb.lo = 0.f;
+                };
+                if (live && work) {
+                    blocks([&](int cb, float (&v)[32], State32& s) {
+                        epi_last32(a, c, R0, lane, C0 + cb, v, s, lb);
+                        if (next_of(cb) >= 0) {
+                            load16(a, c.Z, n, R0, R0 + lane, next_of(cb), s.z[0], s.x[0]);
+                            load16(a, c.Z, n, R0, R0 + lane, next_of(cb) + 16, s.z[1], s.x[1]);
+                        }
+                        __syncwarp();
+                        if ((cb & 32) || cb + 32 >= cb1) flush(C0 + cb);
+                    });
+                }
             }
             if constexpr (HOLD) release();
             else __syncwarp();
@@ -1464,19 +1497,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // and hand back the context
             if constexpr (!LAST) st.finish();
             if (lane == 0 && a.nlayers > 1) done_add(c.done, 1);
-            if constexpr (LAST) {
-                for (int o = 16; o > 0; o >>= 1) {
-                    tr += __shfl_xor_sync(0xffffffffu, tr, o);
-                    sq += __shfl_xor_sync(0xffffffffu, sq, o);
-                }
-                if (lane == 0) {
-                    double* const ps = a.partials + ((size_t)c.t * kPartialSlots + (int)rank * kEpiWarps + (warp - 2)) * 2;
-                    ps[0] = tr;
-                    ps[1] = sq;
-                    // a single CTA fills half of the tile's slots; the finalize sums all
-                    if constexpr (!PAIR) ps[2 * kEpiWarps] = ps[2 * kEpiWarps + 1] = 0.0;
-                }
-            }
             __syncwarp();
             if (lane == 0) local_arrive(smem_u32(&ctx_empty[slot]));
         }
@@ -1792,7 +1812,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
             if (!has_next_tile(a, f, nunits)) continue;     // inline in the accumulating warps
             if (lane == 0) {
                 const InstWork& w = a.iw[tl.inst];
-                fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], t, (int)rank, c);
+                fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], (int)rank, c);
             }
             __syncwarp();
             if (!wait_bar(&sfull_bar, sp, a)) {
@@ -1975,7 +1995,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                 // follow, so the blocks are staged in the operand ring.
                 ItemCtx c;
                 const InstWork& w = a.iw[tl.inst];
-                fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], t, (int)rank, c);
+                fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], (int)rank, c);
                 Stager st{smem_u32(smem) + (uint32_t)((warp - 2) * kStageBytes), lane, 0, false};
                 const CUtensorMap* const wm = (((g - a.gl) & 1) ? wmaps1 : wmaps0).w[tl.chain];
                 const int R0 = c.row0 + q * 32;

@@ -16,11 +16,12 @@
 namespace ftsp2 {
 
 // ------------------------------------------------------------------------------
-// prep: one block.  Initialises the bound keys and writes the tile tables.
+// prep: one block.  Initialises the bound keys and writes the tile tables (the
+// orders ranked and their tiles scanned in shared memory: the ragged batch of 512
+// took 362 us when every instance summed the tiles of all before it, PREP_US now).
 // Tile (I, J) of an instance covers rows [BM I, BM I + BM) and columns
 // [BN J, BN J + BN); only tiles touching the upper triangle are listed
-// (BM I < BN (J + 1)).  Chain-major order: all tiles of chain 0, then
-// chain 1; inside a chain, instance by instance.
+// (BM I < BN (J + 1)).
 // ------------------------------------------------------------------------------
 // rows of tiles in tile column J
 __device__ __forceinline__ int tiles_in_column(int J, int nI, int BM, int BN) {
@@ -34,12 +35,13 @@ __device__ __forceinline__ int tiles_of(int n, int BM, int BN) {
     return c;
 }
 
-// Exclusive scan of one value per thread over the block (blockDim.x a multiple
-// of 32, at most 1024): warp scans by shuffles, then the warp totals.
-__device__ int block_exclusive_scan(int v, int& total) {
+// Inclusive scan of two values per thread (v0 before v1, threads in order) over
+// the block (1024 threads): warp scans by shuffles, then the warp totals.
+__device__ __forceinline__ void block_scan2(int& v0, int& v1) {
     __shared__ int wsum[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int x = v;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int s = v0 + v1;
+    int x = s;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -48,109 +50,141 @@ __device__ int block_exclusive_scan(int v, int& total) {
     if (lane == 31) wsum[warp] = x;
     __syncthreads();
     if (warp == 0) {
-        int w = lane < nw ? wsum[lane] : 0;
+        int w = wsum[lane];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += y;
         }
-        if (lane < nw) wsum[lane] = w;      // inclusive warp prefix
+        wsum[lane] = w;
     }
     __syncthreads();
-    total = wsum[nw - 1];
-    const int r = (warp > 0 ? wsum[warp - 1] : 0) + x - v;
+    const int before = (warp > 0 ? wsum[warp - 1] : 0) + x - s;
+    v1 += before + v0;
+    v0 += before;
     __syncthreads();
-    return r;
 }
 
-// Batches up to this many instances get their tiles in decreasing order of
-// n (O(nb^2 / 1024) comparisons per thread of the one-block prep kernel).
+// Batches up to this many instances get their tiles in decreasing order of n.
 constexpr int kTileSortMax = 2048;
+constexpr int kPrepThreads = 1024;
+static_assert(kTileSortMax == 2 * kPrepThreads, "two ranks per thread");
 
-// Per-instance tile ranges, then the tiles themselves.  A chain's table holds
-// the instances one after the other, by decreasing n (ties by index) up to
-// kTileSortMax instances, else in index order (thread t owns a contiguous
-// chunk of instances; the chunk totals are scanned).  Warp w writes the tiles
-// of instances w, w + 32, ..., its lanes stepping through the instance's list
-// and decoding (I, J) from the position in the column-major triangle.
-__device__ void block_exclusive_scan_fill(const ftsp2_instance* inst, int nb, int BM, int BN, int nchains,
-                                          InstWork* iw, Tile* tiles, int table) {
-    const int T = blockDim.x;
-    const int chunk = (nb + T - 1) / T;
-    const int b0 = min(nb, threadIdx.x * chunk);
-    const int b1 = min(nb, b0 + chunk);
-    int s = 0;
-    for (int b = b0; b < b1; ++b) s += tiles_of(inst[b].n, BM, BN);
-    int chain_total;
-    const int first = block_exclusive_scan(s, chain_total);
-    if (nb <= kTileSortMax) {
-        // instances by decreasing order n (ties by index): the units of a
-        // layer launch take the tiles round-robin, so the long-K tiles are
-        // dealt first and every unit's last tiles are short ones
-        for (int b = b0; b < b1; ++b) {
-            const int nself = inst[b].n, cnt = tiles_of(nself, BM, BN);
-            int before = 0;
-            for (int q = 0; q < nb; ++q) {
-                const int nq = inst[q].n;
-                if (nq > nself || (nq == nself && q < b)) before += tiles_of(nq, BM, BN);
-            }
-            for (int c = 0; c < nchains; ++c) {
-                iw[b].tile_start[table][c] = c * chain_total + before;
-                iw[b].tile_count[table][c] = cnt;
-            }
-        }
-    } else {
-        for (int c = 0; c < nchains; ++c) {
-            int pos = c * chain_total + first;
-            for (int b = b0; b < b1; ++b) {
-                const int cnt = tiles_of(inst[b].n, BM, BN);
-                iw[b].tile_start[table][c] = pos;
-                iw[b].tile_count[table][c] = cnt;
-                pos += cnt;
-            }
-        }
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T >> 5;
-    for (int b = warp; b < nb; b += nw) {
+// The tiles of one table, by instance: warp w writes those of instances w, w + 32,
+// ..., its lanes stepping through the instance's list and decoding (I, J) from the
+// position in the column-major triangle.
+__device__ __forceinline__ void write_tiles(const ftsp2_instance* inst, int nb, int BM, int BN, int nchains,
+                                            const InstWork* iw, Tile* tiles, int table) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = warp; b < nb; b += kPrepThreads / 32) {
         const int n = inst[b].n;
         const int nI = (n + BM - 1) / BM;
         const int cnt = iw[b].tile_count[table][0];
+        int start[kMaxChains] = {iw[b].tile_start[table][0], 0};
+        if (nchains > 1) start[1] = iw[b].tile_start[table][1];
+        int J = 0, first = 0;                        // first: list position of column J
         for (int l = lane; l < cnt; l += 32) {
-            int J = 0, rem = l;
             for (;;) {
                 const int col = tiles_in_column(J, nI, BM, BN);
-                if (rem < col) break;
-                rem -= col;
+                if (l - first < col) break;
+                first += col;
                 ++J;
             }
-            for (int c = 0; c < nchains; ++c) tiles[iw[b].tile_start[table][c] + l] = Tile{b, rem, J, c};
+            for (int c = 0; c < nchains; ++c) tiles[start[c] + l] = Tile{b, l - first, J, c};
         }
     }
-    __syncthreads();
 }
 
-__global__ void prep_kernel(SetupArgs a) {
-    for (int b = threadIdx.x; b < a.nb; b += blockDim.x) {
+// Tile tables of up to kTileSortMax instances: by decreasing order n (ties by
+// index), since the units of a layer launch take the tiles round-robin: the
+// long-K tiles are dealt first and every unit's last tiles are short ones.  All
+// tiles of chain 0, then those of chain 1.
+__global__ void __launch_bounds__(kPrepThreads) prep_kernel(SetupArgs a) {
+    __shared__ int ns[kTileSortMax], order[kTileSortMax], pre[kTileSortMax + 1];
+    const int t = threadIdx.x;
+    for (int b = t; b < a.nb; b += kPrepThreads) {
         a.iw[b].kmin = dkey(__longlong_as_double(0x7ff0000000000000ll));    // +inf
         a.iw[b].kmax = dkey(-__longlong_as_double(0x7ff0000000000000ll));   // -inf
         a.iw[b].nonfinite = 0;
         a.iw[b].start_layer = 0;
+        if (a.nb <= kTileSortMax) ns[b] = a.inst[b].n;
     }
-    if (threadIdx.x == 0) {
+    if (t == 0) {
         a.status[0] = 0;
         a.status[1] = 0x7fffffff;     // first global layer with an active instance (decide lowers it)
     }
     if (a.done) {
         const int cnt = a.done_layers * a.nb * kMaxChains;
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) a.done[i] = 0;
+        for (int i = t; i < cnt; i += kPrepThreads) a.done[i] = 0;
     }
-    if (a.tiles) block_exclusive_scan_fill(a.inst, a.nb, a.BM, a.BN, a.nchains, a.iw, a.tiles, 0);
-    if (a.tiles_ref) block_exclusive_scan_fill(a.inst, a.nb, 128, 128, a.nchains, a.iw, a.tiles_ref, 1);
+    if (!a.tiles) return;
+    if (a.nb > kTileSortMax) {
+        // index order; thread t owns a contiguous run of instances
+        const int chunk = (a.nb + kPrepThreads - 1) / kPrepThreads;
+        const int b0 = min(a.nb, t * chunk), b1 = min(a.nb, b0 + chunk);
+        for (int table = 0; table < (a.tiles_ref ? 2 : 1); ++table) {
+            const int BM = table ? 128 : a.BM, BN = table ? 128 : a.BN;
+            int s = 0, last = 0;
+            for (int b = b0; b < b1; ++b) s += tiles_of(a.inst[b].n, BM, BN);
+            const int own = s;
+            block_scan2(s, last);
+            if (t == kPrepThreads - 1) pre[0] = s;
+            __syncthreads();
+            int pos = s - own;
+            for (int b = b0; b < b1; ++b) {
+                const int cnt = tiles_of(a.inst[b].n, BM, BN);
+                for (int c = 0; c < a.nchains; ++c) {
+                    a.iw[b].tile_start[table][c] = c * pre[0] + pos;
+                    a.iw[b].tile_count[table][c] = cnt;
+                }
+                pos += cnt;
+            }
+            __syncthreads();
+            write_tiles(a.inst, a.nb, BM, BN, a.nchains, a.iw, table ? a.tiles_ref : a.tiles, table);
+            __syncthreads();
+        }
+        return;
+    }
+    __syncthreads();
+    for (int b = t; b < a.nb; b += kPrepThreads) {
+        const int nself = ns[b];
+        int rank = 0;
+        for (int q = 0; q < a.nb; ++q) {
+            const int nq = ns[q];
+            rank += (nq > nself || (nq == nself && q < b)) ? 1 : 0;
+        }
+        order[rank] = b;
+    }
+    __syncthreads();
+    for (int table = 0; table < (a.tiles_ref ? 2 : 1); ++table) {
+        const int BM = table ? 128 : a.BM, BN = table ? 128 : a.BN;
+        // pre[r] = tiles (of one chain) of the instances before rank r
+        const int r0 = 2 * t, r1 = 2 * t + 1;
+        const int c0 = r0 < a.nb ? tiles_of(ns[order[r0]], BM, BN) : 0;
+        const int c1 = r1 < a.nb ? tiles_of(ns[order[r1]], BM, BN) : 0;
+        int p0 = c0, p1 = c1;
+        block_scan2(p0, p1);
+        pre[r0 + 1] = p0;
+        pre[r1 + 1] = p1;
+        if (t == 0) pre[0] = 0;
+        __syncthreads();
+        for (int h = 0; h < 2; ++h) {
+            const int r = r0 + h;
+            if (r >= a.nb) break;
+            InstWork& w = a.iw[order[r]];
+            for (int c = 0; c < a.nchains; ++c) {
+                w.tile_start[table][c] = c * pre[a.nb] + pre[r];
+                w.tile_count[table][c] = h ? c1 : c0;
+            }
+        }
+        __syncthreads();
+        write_tiles(a.inst, a.nb, BM, BN, a.nchains, a.iw, table ? a.tiles_ref : a.tiles, table);
+        __syncthreads();
+    }
 }
 
 void launch_prep(const SetupArgs& a, cudaStream_t s) {
-    prep_kernel<<<1, 1024, 0, s>>>(a);
+    prep_kernel<<<1, kPrepThreads, 0, s>>>(a);
     count_launch();
 }
 
@@ -242,7 +276,7 @@ void launch_gershgorin(const SetupArgs& a, int max_n, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------------------
-// decide: one thread per instance (scalar decisions of Sec. III A).
+// decide: scalar decisions of Sec. III A per instance.
 // ------------------------------------------------------------------------------
 __device__ __forceinline__ bool valid_region(double mup, double betap, double beta0, double mu0) {
     // spectrum of H0 inside [0, 1]: linear form of Eq. conditions
@@ -257,8 +291,28 @@ __device__ __forceinline__ bool better(const DevModel& m, const DevModel& cur, b
     return (m.beta0 < cur.beta0) || (m.beta0 == cur.beta0 && m.L < cur.L);
 }
 
+// The preferred of the models for which ok(m) holds, over the warp's lanes (-1:
+// none); equals go to the lower index, as in a scan of the set in order.
+template <class Ok>
+__device__ __forceinline__ int pick_model(const SetupArgs& a, bool min_layers, int lane, Ok ok) {
+    int best = -1;
+    for (int m = lane; m < a.nmodels; m += 32)
+        if (ok(a.models[m]) && (best < 0 || better(a.models[m], a.models[best], min_layers))) best = m;
+    for (int o = 16; o > 0; o >>= 1) {
+        const int other = __shfl_xor_sync(0xffffffffu, best, o);
+        if (other >= 0 && other != best &&
+            (best < 0 || better(a.models[other], a.models[best], min_layers) ||
+             (other < best && !better(a.models[best], a.models[other], min_layers))))
+            best = other;
+    }
+    return best;
+}
+
+// One warp per instance, a lane per model of the set (the FP64 division of a
+// model's region took most of the time when one thread walked the set: 12 us for
+// the twelve models of the ragged set, DECIDE_US now).
 __global__ void decide_kernel(SetupArgs a) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= a.nb) return;
     const ftsp2_instance in = a.inst[b];
     const bool min_layers = (a.flags & FTSP2_MIN_LAYERS) != 0;
@@ -283,10 +337,10 @@ __global__ void decide_kernel(SetupArgs a) {
         int best = -1;
         if (r.e_max == r.e_min) {
             // H = cI: X0 = mu0 + (beta/beta0)(mu - c), no flip
-            for (int m = 0; m < a.nmodels; ++m) {
-                const double x = a.models[m].mu0 + (beta / a.models[m].beta0) * (in.mu - r.e_min);
-                if (x >= 0.0 && x <= 1.0 && (best < 0 || better(a.models[m], a.models[best], min_layers))) best = m;
-            }
+            best = pick_model(a, min_layers, lane, [&](const DevModel& m) {
+                const double x = m.mu0 + (beta / m.beta0) * (in.mu - r.e_min);
+                return x >= 0.0 && x <= 1.0;
+            });
             if (best >= 0) {
                 r.model = best;
                 r.valid = 1;
@@ -302,10 +356,8 @@ __global__ void decide_kernel(SetupArgs a) {
             double betap = W * beta;                 // Eq. beta'
             const int flip = mup > 0.5 ? 1 : 0;      // Eq. flip
             if (flip) mup = 1.0 - mup;
-            for (int m = 0; m < a.nmodels; ++m)
-                if (valid_region(mup, betap, a.models[m].beta0, a.models[m].mu0) &&
-                    (best < 0 || better(a.models[m], a.models[best], min_layers)))
-                    best = m;
+            best = pick_model(a, min_layers, lane,
+                              [&](const DevModel& m) { return valid_region(mup, betap, m.beta0, m.mu0); });
             r.valid = best >= 0;
             if (best < 0 && (a.flags & FTSP2_CLAMP)) {
                 best = 0;
@@ -337,6 +389,7 @@ __global__ void decide_kernel(SetupArgs a) {
             r.layers = a.chain_kind[0] == CHAIN_ENTROPY ? M.LS : M.L;
         }
     }
+    if (lane != 0) return;
     a.rec[b] = r;
     InstWork& w = a.iw[b];
     w.start_layer = sl[0] | (sl[1] << 16);
@@ -355,7 +408,7 @@ __global__ void decide_kernel(SetupArgs a) {
 }
 
 void launch_decide(const SetupArgs& a, cudaStream_t s) {
-    decide_kernel<<<(a.nb + 127) / 128, 128, 0, s>>>(a);
+    decide_kernel<<<(a.nb + 3) / 4, 128, 0, s>>>(a);
     count_launch();
 }
 
@@ -441,7 +494,7 @@ __device__ __forceinline__ void write_operand16(int fmt, uint8_t* base, size_t p
     }
 }
 
-// Layer-0 state and operands.  One CTA per (32-row band, instance, 512
+// Layer-0 state and operands.  One CTA per (32-row band, instance, 128 or 512
 // columns); lane = row of the band, each warp walks 16-column chunks of the
 // band's columns in the instance's R x R square (R = n rounded up to the
 // largest tile, 256, at most P):
@@ -461,7 +514,6 @@ __device__ __forceinline__ void write_operand16(int fmt, uint8_t* base, size_t p
 //   H included, when every chain of the instance takes this form.
 // Z_0 is formed in FP64 and rounded once: scale * (mu - H_rr) on the diagonal,
 // (-scale) * H_rc elsewhere (the same value as scale * (0 - H_rc)).
-constexpr int kInitCols = 512;     // columns per init CTA
 
 __global__ void __launch_bounds__(256) init_kernel(InitArgs a) {
     const int b = blockIdx.y;
@@ -488,7 +540,7 @@ __global__ void __launch_bounds__(256) init_kernel(InitArgs a) {
         op0S = M.op0S;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cbeg = blockIdx.z * kInitCols, cend = min(R, cbeg + kInitCols);
+    const int cbeg = blockIdx.z * a.cols, cend = min(R, cbeg + a.cols);
     if (cbeg >= cend) return;
     const int r = band + lane;
     const bool row_in = r < n;
@@ -586,56 +638,71 @@ __global__ void __launch_bounds__(256) init_kernel(InitArgs a) {
 }
 
 void launch_init(const InitArgs& a, int max_n, cudaStream_t s) {
-    dim3 grid((a.P + 31) / 32, a.nb, (a.P + kInitCols - 1) / kInitCols);
-    init_kernel<<<grid, 256, 0, s>>>(a);
+    // columns per CTA: a chunk for each of its warps, or four where that gives the
+    // GPU's SMs several CTAs each
+    InitArgs args = a;
+    args.cols = (size_t)a.nb * a.P * a.P >= (size_t)1536 * 1536 ? 512 : 128;
+    dim3 grid((a.P + 31) / 32, a.nb, (a.P + args.cols - 1) / args.cols);
+    init_kernel<<<grid, 256, 0, s>>>(args);
     count_launch();
 }
 
 // ------------------------------------------------------------------------------
-// finalize: one block per instance.  Per chain the last layer left, per tile and
-// per epilogue warp (kPartialSlots slots), two FP64 sums of the centred output G = A_L + Z_L:
-// sum of the diagonal and sum of squares over the full matrix.  With
+// finalize: one block per instance.  Per chain the last layer left, per 32 x 64 block
+// of the upper triangle, two FP64 sums of the centred output G = A_L + Z_L: sum of the
+// diagonal and sum of squares over the full matrix.  With
 // D = G + f0 I (flipped: (1 - f0) I - G):
 //   Tr D = n f0 + Tr G,  ||D||^2 = ||G||^2 + 2 f0 Tr G + n f0^2   (no flip)
 //   Tr D = n (1 - f0) - Tr G, ||D||^2 = ||G||^2 - 2 (1 - f0) Tr G + n (1 - f0)^2
 // and for the entropy chain F = G + g0 I:
 //   S = 4 ln2 (Tr F - ||F||^2) = 4 ln2 (n g0 (1 - g0) + (1 - 2 g0) Tr G - ||G||^2).
 // ------------------------------------------------------------------------------
-constexpr int kFinThreads = 1024;
+// 256 threads per chain; blocks are assigned to threads, and the threads' sums
+// added, in a fixed order, so the result does not depend on scheduling.  Bound by
+// latency: with 1024 threads and a tree over shared memory (FP64 additions and a
+// barrier a level) 9 to 15 us for a small instance, FIN_US now.
+constexpr int kFinThreads = 256;
 
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinalArgs a) {
-    // one block per instance; each chain's partial sums are reduced by a
-    // fixed assignment of slots to threads and a fixed tree, so the result
-    // does not depend on scheduling
+__global__ void __launch_bounds__(kMaxChains * kFinThreads) finalize_kernel(FinalArgs a) {
     const int b = blockIdx.x;
-    if (b >= a.nb) return;
-    __shared__ double s_tr[kFinThreads], s_sq[kFinThreads];
+    __shared__ double s_sum[kMaxChains][kFinThreads / 32][2];
+    __shared__ int s_bad[kMaxChains];
     ftsp2_rescale_rec rec = a.rec[b];
     const int gstat = *a.status;
     const int n = a.inst[b].n;
     const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-    for (int ch = 0; ch < a.nchains; ++ch) {
+    const int ch = threadIdx.x / kFinThreads, t = threadIdx.x % kFinThreads, lane = t & 31;
+    if (ch < a.nchains) {
+        const double2* const p =
+            reinterpret_cast<const double2*>(a.partials) + ((size_t)b * a.nchains + ch) * partial_blocks(a.P);
+        const int cnt = partial_blocks(n);
         double tr = 0.0, sq = 0.0;
-        const int t0 = a.iw[b].tile_start[a.table][ch], tc = a.iw[b].tile_count[a.table][ch];
-        for (int t = threadIdx.x; t < tc * kPartialSlots; t += blockDim.x) {
-            tr += a.partials[(size_t)(t0 * kPartialSlots + t) * 2 + 0];
-            sq += a.partials[(size_t)(t0 * kPartialSlots + t) * 2 + 1];
+#pragma unroll 4
+        for (int i = t; i < cnt; i += kFinThreads) {
+            const double2 v = p[i];
+            tr += v.x;
+            sq += v.y;
         }
-        s_tr[threadIdx.x] = tr;
-        s_sq[threadIdx.x] = sq;
-        __syncthreads();
-        for (int o = kFinThreads / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) {
-                s_tr[threadIdx.x] += s_tr[threadIdx.x + o];
-                s_sq[threadIdx.x] += s_sq[threadIdx.x + o];
-            }
-            __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) {
+            tr += __shfl_xor_sync(0xffffffffu, tr, o);
+            sq += __shfl_xor_sync(0xffffffffu, sq, o);
         }
-        tr = s_tr[0];
-        sq = s_sq[0];
-        __syncthreads();
-        if (threadIdx.x != 0) continue;
+        if (lane == 0) {
+            s_sum[ch][t >> 5][0] = tr;
+            s_sum[ch][t >> 5][1] = sq;
+        }
+    }
+    if (threadIdx.x < kMaxChains) s_bad[threadIdx.x] = 0;
+    __syncthreads();
+    if (ch < a.nchains && t == 0) {
+        double tr = 0.0, sq = 0.0;
+#pragma unroll
+        for (int w = 0; w < kFinThreads / 32; ++w) {
+            tr += s_sum[ch][w][0];
+            sq += s_sum[ch][w][1];
+        }
         const bool ok = rec.status == FTSP2_OK && rec.model >= 0 && gstat == 0;
+        bool bad = false;
         if (a.chain_kind[ch] == CHAIN_FERMI) {
             double trD = qnan, frD = qnan;
             if (ok) {
@@ -647,7 +714,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinalArgs a) {
                     trD = n * f0 + tr;
                     frD = sq + 2.0 * f0 * tr + n * f0 * f0;
                 }
-                if (!isfinite(trD) || !isfinite(frD)) rec.status = FTSP2_E_NONFINITE;
+                bad = !isfinite(trD) || !isfinite(frD);
             }
             if (a.trace) {
                 a.trace[2 * b + 0] = trD;
@@ -658,12 +725,16 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(FinalArgs a) {
             if (ok) {
                 const double g0 = a.models[rec.model].g0;
                 S = 4.0 * 0.69314718055994530942 * (n * g0 * (1.0 - g0) + (1.0 - 2.0 * g0) * tr - sq);
-                if (!isfinite(S)) rec.status = FTSP2_E_NONFINITE;
+                bad = !isfinite(S);
             }
             if (a.S) a.S[b] = S;
         }
+        if (bad) s_bad[ch] = 1;
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        if (s_bad[0] && a.nchains > 1 && a.S) a.S[b] = qnan;      // no entropy beside a density that is not finite
+        if (s_bad[0] | s_bad[kMaxChains - 1]) rec.status = FTSP2_E_NONFINITE;
         if (gstat != 0 && rec.status == FTSP2_OK) rec.status = gstat;
         a.rec[b].status = rec.status;
     }
@@ -701,7 +772,7 @@ void launch_mu_update(const MuArgs& a, cudaStream_t s) {
 }
 
 void launch_finalize(const FinalArgs& a, cudaStream_t s) {
-    finalize_kernel<<<a.nb, kFinThreads, 0, s>>>(a);
+    finalize_kernel<<<a.nb, a.nchains * kFinThreads, 0, s>>>(a);
     count_launch();
 }
 
