@@ -42,18 +42,21 @@
 // max|D - D_ref| = 1.85e-6 / 9.0e-7 / 6.9e-7 at layer times 0.235 / 0.251 /
 // 0.314 ms (an earlier kernel); 128 is the default.
 //
-// layer_tc_kernel (352 threads per CTA, up to 168 registers; persistent over the
-// unit's items):
+// layer_tc_kernel (persistent over the unit's items):
 //   warp 0     : TMA producer (ring of 128-byte K-slices)
 //   warp 1     : TMEM allocation; MMA issuer (even CTA)
-//   warps 2..9 : epilogue warps; warp w reads TMEM lane quarter w % 4 and column
-//                half (w - 2) / 4 of the CTA's 128-row accumulator, adds the chunks
-//                in FP32 registers and runs the final epilogue (Z_{k+1}, A_{k+1},
-//                next operands).  With 16 warps of 96 registers the same work
-//                spilled, and bound by instruction issue (some 60 instructions an
-//                element) a 128 x 128 tile's final epilogue took 8000 to 12000
-//                clocks; 4400 to 6700 now
-//   warp 10    : context warp (below)
+//   warps 2 .. : epilogue warps; warp w reads TMEM lane quarter w % 4 and a column
+//                group of the CTA's 128-row accumulator, adds the chunks in FP32
+//                registers and runs the final epilogue (Z_{k+1}, A_{k+1}, next
+//                operands).  It is a chain of short dependent steps (a warp issues
+//                an instruction every eleven clocks), so FP16X2 operands of
+//                128-column tiles have 16 warps of 32 columns (96 registers) and
+//                the others 8 warps of 64 or 128 columns (168 registers): the
+//                wider formats' planes do not fit in 96.  8 -> 16 warps, FP16X2:
+//                n = 256 277 -> 261 us, 60 fragments 411 -> 380, ragged batch
+//                22.8 -> 22.1 ms, n = 1501 unchanged; BF16X3 and TF32X3 0.7 %
+//                slower at n = 1024 and 2048.
+//   last warp  : context warp (below)
 // The loops of warps 0 and 1 run on the whole warp with one elected lane issuing:
 // their values are then uniform, and a copy or an MMA takes no moves from vector
 // registers to uniform ones (110 against 71 clocks per 128-column MMA, 150
@@ -136,9 +139,11 @@ struct Geo {
     static constexpr int NBUF = 512 / TN;
 };
 constexpr int kCtaRows = 128;
-constexpr int kEpiWarps = 8;
-constexpr int kCtxWarp = 2 + kEpiWarps;            // context warp (layer_tc_kernel)
-constexpr int kTcThreads = 32 * (kCtxWarp + 1);
+// Epilogue warps of layer_tc_kernel, followed by the context warp.
+template <int OUTFMT, int SHAPE>
+constexpr int epi_warps() { return OUTFMT == OP_F16X2 && SHAPE != SHAPE_PAIR ? 16 : 8; }
+template <int OUTFMT, int SHAPE>
+constexpr int tc_threads() { return 32 * (2 + epi_warps<OUTFMT, SHAPE>() + 1); }
 // Deferred final epilogue: store warps, their shared-memory staging ring
 // (entries of 16 columns x 32 rows: sums, Z_k, A_k) and the per-CTA scratch
 // of finished tile sums in global memory (one 32-row x 64-column block per
@@ -581,7 +586,8 @@ struct __align__(16) ItemCtx {
 // (c, r); a block on the diagonal is made symmetric in shared memory.  Rows and
 // columns from n on are written as zeros.  The TMA unit writes 32 bytes a clock:
 // 2000 clocks for the 64 KB of a 128 x 128 tile's FP16X2 operands.
-constexpr int kStageBytes = 4096;                // operand staging of an epilogue warp
+constexpr int kStageBytes = 4096;                // operand staging of a store warp
+constexpr int kStagingBytes = 32768;             // ... of the epilogue warps of layer_tc_kernel
 constexpr int kStateZ = 256, kStateA = 384;      // TMEM columns of a resident tile's state
 
 // State of row r, columns c .. c + 15 (c % 16 == 0): the 8-column groups below the
@@ -641,24 +647,22 @@ struct PlaneWords {
 
 // The warp's staging: boxes of 32 rows x 64 bytes, written in turn, in the layout
 // of TMA's 64-byte swizzle (the 16-byte chunk index is XORed with bits 1-2 of the
-// row).  Two boxes of its own, or, where the unit keeps one tile for all layers,
-// kRingBoxes in the operand ring: its MMAs have all completed when the epilogue
+// row).  One or two boxes of its own, or, where the unit keeps one tile for all
+// layers, its share of kRingBytes in the operand ring: its MMAs have all completed when the epilogue
 // starts, and the loads of the next layer wait for the completions that the
 // epilogue warps count after their stores.
-constexpr int kRingBoxes = 9;                        // 18 KB for each warp of a 144 KB ring
+constexpr int kRingBytes = 144 * 1024;
 struct Stager {
     uint32_t base;                                   // boxes of 2 KB, 1024-byte aligned
     int lane, used;                                  // lane; boxes sent so far
-    bool many;                                       // kRingBoxes boxes (else 2)
-    __device__ __forceinline__ uint32_t box() const {
-        return base + (uint32_t)(many ? used % kRingBoxes : used & 1) * 2048u;
-    }
+    int cap;                                         // boxes
+    __device__ __forceinline__ uint32_t box() const { return base + (uint32_t)(used % cap) * 2048u; }
     // the next box may be written: the store that last used it has read it
     __device__ __forceinline__ void next() const {
-        if (used < (many ? kRingBoxes : 2)) return;
+        if (used < cap) return;
         if (lane == 0) {
-            if (many) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            else asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            if (cap == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
         __syncwarp();
     }
@@ -737,60 +741,66 @@ __device__ __forceinline__ void store_plane(const CUtensorMap* map, Stager& st, 
     }
 }
 
-// The state of 32 columns of a row, loaded ahead.
-struct State32 {
-    float z[2][16], x[2][16];
+// The state of 16 H columns of a row, loaded ahead.
+template <int H>
+struct State {
+    float z[H][16], x[H][16];
 };
+using State32 = State<2>;
 
 // One 32 x 32 block: v holds the sums S of the lane's row.
-template <int FMT, bool CAN_RESIDE>
+template <int FMT, bool CAN_RESIDE, int H>
 __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c, const CUtensorMap* wmaps, Stager& st,
                                             int R0, int c0, uint32_t tstate, bool from_tmem, bool to_tmem,
-                                            float (&v)[32], State32& s, int c_next) {
+                                            float (&v)[32], State<H>& s, int c_next) {
     constexpr int NPL = OpFmtT<FMT>::NPL;
     const int n = c.n, r = R0 + st.lane;
     const float mul = c.mul, bp = c.bp, d = c.d;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int cc = c0 + 16 * h;
+        const int cc = c0 + 16 * h, hs = H == 2 ? h : 0;
         if (cc < n) {
             if (CAN_RESIDE && from_tmem) {
-                tmem_ld16(tstate + 16 * h, reinterpret_cast<uint32_t*>(s.z[h]));
-                tmem_ld16(tstate + (kStateA - kStateZ) + 16 * h, reinterpret_cast<uint32_t*>(s.x[h]));
+                tmem_ld16(tstate + 16 * h, reinterpret_cast<uint32_t*>(s.z[hs]));
+                tmem_ld16(tstate + (kStateA - kStateZ) + 16 * h, reinterpret_cast<uint32_t*>(s.x[hs]));
                 tmem_wait_ld();
             }
             if (c.simple) {
                 // Eq. mlsp2: d2 = 0, p = 1, q = 0
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
-                    v[16 * h + u] = fmaf(mul, v[16 * h + u], bp * s.z[h][u]);
-                    s.x[h][u] = fmaf(d, s.z[h][u], s.x[h][u]);
+                    v[16 * h + u] = fmaf(mul, v[16 * h + u], bp * s.z[hs][u]);
+                    s.x[hs][u] = fmaf(d, s.z[hs][u], s.x[hs][u]);
                 }
             } else {
                 const float d2 = c.d2, p1 = c.p, q1 = c.q;
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
-                    const float xh = fmaf(mul, v[16 * h + u], bp * s.z[h][u]);
-                    const float an = fmaf(d2, xh, fmaf(d, s.z[h][u], s.x[h][u]));
-                    v[16 * h + u] = fmaf(p1, xh, q1 * s.x[h][u]);
-                    s.x[h][u] = an;
+                    const float xh = fmaf(mul, v[16 * h + u], bp * s.z[hs][u]);
+                    const float an = fmaf(d2, xh, fmaf(d, s.z[hs][u], s.x[hs][u]));
+                    v[16 * h + u] = fmaf(p1, xh, q1 * s.x[hs][u]);
+                    s.x[hs][u] = an;
                 }
             }
             if (CAN_RESIDE && to_tmem) {
                 tmem_st16(tstate + 16 * h, v + 16 * h);
-                tmem_st16(tstate + (kStateA - kStateZ) + 16 * h, s.x[h]);
+                tmem_st16(tstate + (kStateA - kStateZ) + 16 * h, s.x[hs]);
             } else if (r < n) {
                 float* const Zg = c.Z + state_off(a.P, r, cc);
                 store_state8(Zg, v + 16 * h);
-                store_state8(Zg + a.plane_elems, s.x[h]);
+                store_state8(Zg + a.plane_elems, s.x[hs]);
                 if (cc + 8 < n) {
                     store_state8(Zg + 256, v + 16 * h + 8);
-                    store_state8(Zg + 256 + a.plane_elems, s.x[h] + 8);
+                    store_state8(Zg + 256 + a.plane_elems, s.x[hs] + 8);
                 }
             }
         }
-        // the same columns of the next block
-        if (!from_tmem && c_next >= 0) load16(a, c.Z, n, R0, r, c_next + 16 * h, s.z[h], s.x[h]);
+        if constexpr (H == 2) {
+            // the same columns of the next block
+            if (!from_tmem && c_next >= 0) load16(a, c.Z, n, R0, r, c_next + 16 * h, s.z[h], s.x[h]);
+        } else if (h == 0 && !from_tmem) {
+            load16(a, c.Z, n, R0, r, c0 + 16, s.z[0], s.x[0]);
+        }
     }
     if (!(R0 + 31 < n && c0 + 31 < n)) {
         // zeros in the padding
@@ -915,9 +925,8 @@ struct Stage {
     // in the ring)
     static constexpr int N = (192 * 1024) / BYTES;
     static constexpr int NMAX = (222 * 1024) / BYTES;
-    static constexpr int SMEM = NMAX * BYTES > N * BYTES + kEpiWarps * kStageBytes
-                                    ? NMAX * BYTES : N * BYTES + kEpiWarps * kStageBytes;
-    static_assert(N * BYTES >= kEpiWarps * kRingBoxes * 2048, "ring staging");
+    static constexpr int SMEM = NMAX * BYTES > N * BYTES + kStagingBytes ? NMAX * BYTES : N * BYTES + kStagingBytes;
+    static_assert(N * BYTES >= kRingBytes, "ring staging");
 };
 
 // Blocks of the deferred epilogue: block e of a tile is the half e & 1 of the
@@ -973,7 +982,7 @@ __device__ __forceinline__ void fill_epilogue(const LayerArgs& a, const Tile& tl
 }
 
 template <int MODE, int OUTFMT, int SHAPE>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
     layer_tc_kernel(const __grid_constant__ LayerArgs a, const __grid_constant__ TmaMaps maps0,
                     const __grid_constant__ TmaMaps maps1, const __grid_constant__ WriteMaps wmaps0,
                     const __grid_constant__ WriteMaps wmaps1) {
@@ -983,7 +992,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     constexpr bool PAIR = G::NCTA == 2;
     constexpr bool LAST = OUTFMT == kLastLayer;
     constexpr int TM = G::TM, TN = G::TN;
-    constexpr int EPI_COLS = TN / (kEpiWarps / 4);     // columns per epilogue warp (128 or 64)
+    constexpr int EW = epi_warps<OUTFMT, SHAPE>(), CTX_WARP = 2 + EW;
+    constexpr int EPI_COLS = TN / (EW / 4);            // columns per epilogue warp
     constexpr int BKE = 128 / C::ESIZE;                // K elements per 128-byte slice
     constexpr int KSTEPS = 4;                          // 128-byte slice / 32 bytes per MMA
     constexpr uint32_t IDESC = make_idesc(C::ATYPE, TM, TN);
@@ -1026,12 +1036,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         for (int s = 0; s < G::NBUF; ++s) {
             mbar_init(&tfull_bar[s], 1);
-            mbar_init(&tempty_bar[s], G::NCTA * kEpiWarps);
+            mbar_init(&tempty_bar[s], G::NCTA * EW);
         }
         for (int s = 0; s < kCtxSlots; ++s) {
             mbar_init(&ctx_full[s], 1);
             // read by the epilogue warps, the producer and, on the even CTA, the MMA issuer
-            mbar_init(&ctx_empty[s], kEpiWarps + 1 + (rank == 0 ? 1 : 0));
+            mbar_init(&ctx_empty[s], EW + 1 + (rank == 0 ? 1 : 0));
         }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
@@ -1058,7 +1068,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == kCtxWarp) {
+    if (warp == CTX_WARP) {
         // ---------------- context warp: the unit's active items ----------------
         // 32 items are looked up at a time, a lane each (a model with few layers
         // starts late: many items of a ragged batch are inactive).
@@ -1103,7 +1113,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         // operands and state written by other CTAs of this launch
                         const bool dep = g > a.gl && k > 0;
                         c.dep = dep ? inst_counter(a, g - 1, tl.inst, tl.chain) : nullptr;
-                        c.target = kEpiWarps * G::NCTA * w.tile_count[a.dtab][tl.chain] + (g == a.stall_layer ? 1 : 0);
+                        c.target = EW * G::NCTA * w.tile_count[a.dtab][tl.chain] + (g == a.stall_layer ? 1 : 0);
                         c.done = inst_counter(a, g, tl.inst, tl.chain);
                         c.first = it == 0;
                         c.final = l == a.nlayers - 1;
@@ -1240,6 +1250,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // and descriptors are then uniform values.  With the loop in a single
             // lane every descriptor went through vector registers, and the issue of
             // a 128-column MMA took 110 clocks for the 64 that it runs.
+            // On single CTAs the completed waits of the next slice (and of the next
+            // chunk's buffer) are seen while this slice's last products are queued:
+            // a completed wait, the choice of the descriptors and a commit each take
+            // 100 to 150 clocks of this warp, 900 a slice where a chunk is one
+            // slice.  Ragged batch 22.12 -> 21.85 ms, 60 fragments 380 -> 373 us;
+            // on pairs, whose producer is rarely a slice ahead, the extra look
+            // cost 1.6 % (n = 1501) and 3.5 % (n = 2048 TF32X3).
             const bool leader = elect_one();
             int stage = 0;
             uint32_t phase = 0;
@@ -1260,24 +1277,26 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int ck = uniform32(c.ck), lowA = uniform32(c.lowA), lowB = uniform32(c.lowB);
                 const bool same = SHAPE == SHAPE_SINGLE && uniform32(c.same) != 0;
                 if (leader) local_arrive(smem_u32(&ctx_empty[slot]));
+                bool have_full = false, have_buf = false;
                 for (int kc = 0; kc < nk && ok; kc += ck) {
-                    if (!all_wait(&tempty_bar[buf], aphase ^ 1u, a)) {
+                    if (!have_buf && !all_wait(&tempty_bar[buf], aphase ^ 1u, a)) {
                         ok = false;
                         break;
                     }
-                    tc_fence_after();
+                    have_buf = false;
                     const uint32_t dt = tm + (uint32_t)(buf * TN);
                     const int kend = min(nk, kc + ck);
+                    const int nbuf_next = buf + 1 == nbuf ? 0 : buf + 1;
+                    const uint32_t aphase_next = nbuf_next == 0 ? aphase ^ 1u : aphase;
                     for (int kb = kc; kb < kend; ++kb) {
-                        if (!all_wait(&full_bar[stage], phase, a)) {
+                        if (!have_full && !all_wait(&full_bar[stage], phase, a)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        // skip mode: the stage holds no new data; the commits below
-                        // keep the protocol
-                        const bool mma = uniform32(*reinterpret_cast<volatile int*>(&abort_flag)) == 0;
-                        // the producer's classification of this K-slice (transposed
+                        // In skip mode the stage holds no new data; its MMAs only keep
+                        // the protocol, their sums are not used.
+                        // The producer's classification of this K-slice (transposed
                         // panels: MN-major operand, K steps of two 1 KB atoms per 64 columns)
                         const bool tA = kb < lowA, tB = kb < lowB;
                         const uint32_t so = (uint32_t)((stage * St::BYTES) >> 4);
@@ -1292,21 +1311,31 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         // small values, so fewer additions land on a large partial sum
                         // (the tensor core's FP32 accumulation is not round-to-nearest).
                         // Measured: 15-30 % smaller errors in D and S at the same speed.
-                        if (leader) {
-                            if (mma) {
+                        auto product = [&](int p) {
 #pragma unroll
-                                for (int q = 0; q < C::NPROD; ++q) {
-                                    const int p = C::NPROD - 1 - q;
-#pragma unroll
-                                    for (int kk = 0; kk < KSTEPS; ++kk) {
-                                        const uint64_t da = baseA + (uint32_t)(prod_a(p) * (St::APLANE >> 4)) + kk * stepA;
-                                        const uint64_t db = baseB + planeB + prod_b(p) * strideB + kk * stepB;
-                                        const uint32_t accum = (kk == 0 && q == 0) ? (kb == kc ? 0u : 1u) : 1u;
-                                        if constexpr (PAIR) umma_pair<C::TF32>(dt, da, db, idesc, accum);
-                                        else umma_one<C::TF32>(dt, da, db, idesc, accum);
-                                    }
-                                }
+                            for (int kk = 0; kk < KSTEPS; ++kk) {
+                                const uint64_t da = baseA + (uint32_t)(prod_a(p) * (St::APLANE >> 4)) + kk * stepA;
+                                const uint64_t db = baseB + planeB + prod_b(p) * strideB + kk * stepB;
+                                const uint32_t accum = (kk == 0 && p == C::NPROD - 1) ? (kb == kc ? 0u : 1u) : 1u;
+                                if constexpr (PAIR) umma_pair<C::TF32>(dt, da, db, idesc, accum);
+                                else umma_one<C::TF32>(dt, da, db, idesc, accum);
                             }
+                        };
+                        if (leader) {
+#pragma unroll
+                            for (int p = C::NPROD - 1; p > 0; --p) product(p);
+                        }
+                        const int stage_next = stage + 1 == nst ? 0 : stage + 1;
+                        const uint32_t phase_next = stage_next == 0 ? phase ^ 1u : phase;
+                        if constexpr (!PAIR) {
+                            have_full = kb + 1 < nk &&
+                                        __all_sync(0xffffffffu, try_wait_cluster(&full_bar[stage_next], phase_next));
+                            if (kb + 1 == kend && kend < nk)
+                                have_buf = __all_sync(0xffffffffu,
+                                                      try_wait_cluster(&tempty_bar[nbuf_next], aphase_next ^ 1u));
+                        }
+                        if (leader) {
+                            product(0);
                             if constexpr (PAIR) umma_commit_pair(smem_u32(&empty_bar[stage]));
                             else umma_commit_one(smem_u32(&empty_bar[stage]));
                             if (kb == kend - 1) {
@@ -1315,16 +1344,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             }
                         }
                         __syncwarp();
-                        if (++stage == nst) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
+                        stage = stage_next;
+                        phase = phase_next;
                     }
                     if (!ok) break;
-                    if (++buf == nbuf) {
-                        buf = 0;
-                        aphase ^= 1u;
-                    }
+                    buf = nbuf_next;
+                    aphase = aphase_next;
                 }
             }
             // Drain: every MMA this warp issued (they write TMEM of both CTAs
@@ -1342,15 +1367,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue (warps 2..9) ----------------
+        // ---------------- epilogue (warps 2 .. 1 + EW) ----------------
         const int q = warp & 3;                  // TMEM lane quarter
-        const int cq = (warp - 2) >> 2;          // column half of the tile
+        const int cq = (warp - 2) >> 2;          // column group of the tile
         // "tempty" barriers of the even CTA (consecutive 8-byte words)
         const uint32_t tempty0 = PAIR ? map_to(smem_u32(&tempty_bar[0]), 0) : smem_u32(&tempty_bar[0]);
         const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cq * EPI_COLS);
-        Stager st{resident ? smem_u32(smem) + (uint32_t)((warp - 2) * (kRingBoxes * 2048))
-                           : smem_u32(smem + St::N * St::BYTES) + (uint32_t)((warp - 2) * kStageBytes),
-                  lane, 0, resident};
+        constexpr int RING_BOXES = kRingBytes / EW / 2048, BOXES = kStagingBytes / EW / 2048;
+        Stager st{resident ? smem_u32(smem) + (uint32_t)((warp - 2) * (RING_BOXES * 2048))
+                           : smem_u32(smem + St::N * St::BYTES) + (uint32_t)((warp - 2) * (BOXES * 2048)),
+                  lane, 0, resident ? RING_BOXES : BOXES};
         int buf = 0;
         uint32_t aphase = 0;
         auto release = [&]() {
@@ -1379,18 +1405,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const bool live = cb0 < cb1;
             const int* const dep = resident ? nullptr : c.dep;
             // the state of the first block, loaded ahead of the last chunk
-            State32 ahead;
+            constexpr int AH = EPI_COLS == 32 ? 1 : 2;
+            State<AH> ahead;
             const bool state_global = live && (!resident || c.first);
-            auto load_first = [&](State32& s) {
-                load16(a, c.Z, n, R0, R0 + lane, C0 + cb0, s.z[0], s.x[0]);
-                load16(a, c.Z, n, R0, R0 + lane, C0 + cb0 + 16, s.z[1], s.x[1]);
+            auto load_first = [&](State<AH>& s) {
+#pragma unroll
+                for (int h = 0; h < AH; ++h) load16(a, c.Z, n, R0, R0 + lane, C0 + cb0 + 16 * h, s.z[h], s.x[h]);
             };
             // Chunk drain: every chunk is added into acc and its buffer released.
             // The 128 columns of a 256-column tile's warp leave no registers for
             // the final epilogue: there the finished sum is written back into the
             // last chunk's buffer, which stays held, and read from it block by
             // block; the MMAs of the next tile meanwhile fill the other buffer.
-            constexpr bool HOLD = EPI_COLS > 64;
+            constexpr bool HOLD = TN > 128;
             float acc[EPI_COLS];
 #pragma unroll
             for (int i = 0; i < EPI_COLS; ++i) acc[i] = 0.f;
@@ -1447,6 +1474,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                 } else {
                     float(&v0)[32] = *reinterpret_cast<float(*)[32]>(acc);
+                    if constexpr (EPI_COLS == 32) {
+                        block(0, v0, ahead);
+                        return;
+                    }
                     float(&v1)[32] = *reinterpret_cast<float(*)[32]>(acc + EPI_COLS - 32);
                     if (cb0 == 0) block(0, v0, ahead);
                     if (cb1 == EPI_COLS) block(EPI_COLS - 32, v1, ahead);
@@ -1456,8 +1487,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if constexpr (!LAST) {
                 if (live && work) {
                     const CUtensorMap* const wm = (c.maps ? wmaps1 : wmaps0).w[c.chain];
-                    blocks([&](int cb, float (&v)[32], State32& s) {
-                        epi_block32<OUTFMT, CAN_RESIDE>(a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem,
+                    blocks([&](int cb, float (&v)[32], State<AH>& s) {
+                        epi_block32<OUTFMT, CAN_RESIDE, AH>(a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem,
                                                         to_tmem, v, s, next_of(cb));
                     });
                     if (CAN_RESIDE && to_tmem) tmem_wait_st();
@@ -1796,7 +1827,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
         // two-deep shared ring with cp.async; the warp computes Z_{k+1} and
         // A_{k+1} and writes the next operands block by block.
         const int sw = warp - 2 - kDeferWarps;
-        Stager st{smem_u32(smem + C::STAGES * STAGE_BYTES) + (uint32_t)(sw * kStageBytes), lane, 0, false};
+        Stager st{smem_u32(smem + C::STAGES * STAGE_BYTES) + (uint32_t)(sw * kStageBytes), lane, 0, 2};
         uint8_t* const ring = smem + C::STAGES * STAGE_BYTES + kStoreWarps * kStageBytes + sw * (kRing * kEntryBytes);
         const float* const scr = a.escr + (size_t)blockIdx.x * kEpiScratchFloats;
         ItemCtx& c = dctx[sw];
@@ -1996,7 +2027,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                 ItemCtx c;
                 const InstWork& w = a.iw[tl.inst];
                 fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], (int)rank, c);
-                Stager st{smem_u32(smem) + (uint32_t)((warp - 2) * kStageBytes), lane, 0, false};
+                Stager st{smem_u32(smem) + (uint32_t)((warp - 2) * kStageBytes), lane, 0, 2};
                 const CUtensorMap* const wm = (((g - a.gl) & 1) ? wmaps1 : wmaps0).w[tl.chain];
                 const int R0 = c.row0 + q * 32;
 #pragma unroll 1
@@ -2046,7 +2077,7 @@ struct Variant {
         if constexpr (DEFER) return layer_defer_kernel<MODE, OUTFMT>;
         else return layer_tc_kernel<MODE, OUTFMT, SHAPE>;
     }
-    static constexpr int threads = DEFER ? kDeferThreads : kTcThreads;
+    static constexpr int threads = DEFER ? kDeferThreads : tc_threads<OUTFMT, SHAPE>();
     static constexpr int smem = 1024 + (DEFER ? TcCfg<MODE>::STAGES * TcCfg<MODE>::NSPLIT * 2 * kCtaRows * 128 +
                                                     kStoreWarps * (kStageBytes + kRing * kEntryBytes)
                                               : Stage<MODE, SHAPE>::SMEM);

@@ -18,7 +18,7 @@ namespace ftsp2 {
 // ------------------------------------------------------------------------------
 // prep: one block.  Initialises the bound keys and writes the tile tables (the
 // orders ranked and their tiles scanned in shared memory: the ragged batch of 512
-// took 362 us when every instance summed the tiles of all before it, PREP_US now).
+// took 362 us when every instance summed the tiles of all before it, 36 us now).
 // Tile (I, J) of an instance covers rows [BM I, BM I + BM) and columns
 // [BN J, BN J + BN); only tiles touching the upper triangle are listed
 // (BM I < BN (J + 1)).
@@ -310,7 +310,7 @@ __device__ __forceinline__ int pick_model(const SetupArgs& a, bool min_layers, i
 
 // One warp per instance, a lane per model of the set (the FP64 division of a
 // model's region took most of the time when one thread walked the set: 12 us for
-// the twelve models of the ragged set, DECIDE_US now).
+// the twelve models of the ragged set, 6 us now).
 __global__ void decide_kernel(SetupArgs a) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= a.nb) return;
@@ -660,7 +660,7 @@ void launch_init(const InitArgs& a, int max_n, cudaStream_t s) {
 // 256 threads per chain; blocks are assigned to threads, and the threads' sums
 // added, in a fixed order, so the result does not depend on scheduling.  Bound by
 // latency: with 1024 threads and a tree over shared memory (FP64 additions and a
-// barrier a level) 9 to 15 us for a small instance, FIN_US now.
+// barrier a level) 9 to 15 us for a small instance, 4 us now.
 constexpr int kFinThreads = 256;
 
 __global__ void __launch_bounds__(kMaxChains * kFinThreads) finalize_kernel(FinalArgs a) {
