@@ -64,6 +64,14 @@ __device__ double block_sum(double v, double* sh) {
     return s;
 }
 
+// w / b with r = 1 / b: one correction of the product (Markstein's division step)
+// instead of a full division, some 20 instructions of the FP64 pipe (16 clocks a
+// warp instruction) each.
+__device__ __forceinline__ double div_by(double w, double b, double r) {
+    const double q = w * r;
+    return fma(fma(-q, b, w), r, q);
+}
+
 __device__ __forceinline__ double* lz_vec(const LanczosArgs& a, int which, int b) {
     double* base = which == 0 ? a.V0 : (which == 1 ? a.V1 : a.W);
     return base + (size_t)b * a.P;
@@ -85,9 +93,15 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_start_kernel(LanczosArgs a
         v0[i] = 0.0;
         s += q * q;
     }
-    const double nrm = sqrt(block_sum(s, sh));
+    s = block_sum(s, sh);
+    __shared__ double norm[2];
+    if (threadIdx.x == 0) {
+        norm[0] = sqrt(s);
+        norm[1] = 1.0 / norm[0];
+    }
+    __syncthreads();
     for (int i = threadIdx.x; i < n; i += kLzThreads) {
-        v1[i] /= nrm;
+        v1[i] = div_by(v1[i], norm[0], norm[1]);
         v32[i] = (float)v1[i];
     }
     if (threadIdx.x == 0) a.state[b] = 0;
@@ -158,22 +172,32 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_update_kernel(LanczosArgs 
         w[i] = wi;
         s += wi * wi;
     }
-    const double beta = sqrt(block_sum(s, sh));
-    double* ab = a.ab + (size_t)b * kLzSteps * 2;
-    const double a1 = j == 0 ? alpha : ab[0];
-    const double b1 = j == 0 ? beta : ab[1];
-    const bool stop = beta <= 1e-12 * (fabs(a1) + b1 + 1.0);
-    float* v32 = a.V32 + (size_t)b * a.P;
-    if (!stop)
-        for (int i = threadIdx.x; i < n; i += kLzThreads) {
-            const double v = w[i] / beta;
-            vn[i] = v;
-            v32[i] = (float)v;
-        }
+    // the square root and the reciprocal once, in one thread: by every thread they
+    // and the divisions below were 2.5 of the 11 us of a step at n = 1728
+    s = block_sum(s, sh);
+    __shared__ double norm[2];
+    __shared__ bool done;
     if (threadIdx.x == 0) {
+        const double beta = sqrt(s);
+        double* ab = a.ab + (size_t)b * kLzSteps * 2;
+        const double a1 = j == 0 ? alpha : ab[0];
+        const double b1 = j == 0 ? beta : ab[1];
+        const bool stop = beta <= 1e-12 * (fabs(a1) + b1 + 1.0);
         ab[2 * j] = alpha;
         ab[2 * j + 1] = beta;
         a.state[b] = (j + 1) | (stop ? kLzStopped : 0);
+        norm[0] = beta;
+        norm[1] = 1.0 / beta;
+        done = stop;
+    }
+    __syncthreads();
+    if (done) return;
+    const double beta = norm[0], rbeta = norm[1];
+    float* v32 = a.V32 + (size_t)b * a.P;
+    for (int i = threadIdx.x; i < n; i += kLzThreads) {
+        const double v = div_by(w[i], beta, rbeta);
+        vn[i] = v;
+        v32[i] = (float)v;
     }
 }
 
@@ -187,10 +211,15 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_update_kernel(LanczosArgs 
 // step (one instance each, at most kLzSmallN^2 floats) stay in L2 instead of
 // streaming the whole batch from HBM 24 times.  Arithmetic as in the
 // multi-block kernels: FP32 products and row sums, FP64 vectors, dot
-// products and norms, reductions in a fixed order.
+// products and norms, reductions in a fixed order.  The vectors' FP64 work is on
+// eight of the 32 warps, square roots and reciprocals in one thread: a warp
+// instruction takes 16 clocks of the FP64 pipe, and by every warp the square root,
+// the divisions and the sums were a tenth of the kernel (ragged batch of 512:
+// 2.62 ms, 2.40 now; the rest is reading the rows that are not cached).
 constexpr int kLzSmallN = 1024;
 constexpr int kLzSmallThreads = 1024;
-constexpr int kLzSmallCacheBytes = 160 * 1024;
+constexpr int kLzSmallCacheBytes = 192 * 1024;
+constexpr int kLzVecThreads = 256;               // threads of the vectors' FP64 work
 
 // The queue of the small-instance kernel, in the partial-sum buffer (which
 // only the multi-block path uses; nb RB doubles hold nb + 1 ints): queue[0]
@@ -219,10 +248,23 @@ __global__ void lanczos_queue_kernel(LanczosArgs a) {
     queue[1 + rank] = b;
 }
 
+// Sum over the first kLzVecThreads threads in fixed order, the same in each; all of
+// them call.  sh: one double a warp, not in use (two alternate between calls).
+__device__ __forceinline__ double vec_sum(double v, double* sh) {
+    constexpr int NV = kLzVecThreads / 32;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    asm volatile("bar.sync 1, %0;" ::"n"(kLzVecThreads) : "memory");
+    v = sh[threadIdx.x % NV];
+    for (int o = NV / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 __global__ void __launch_bounds__(kLzSmallThreads, 1) lanczos_small_kernel(LanczosArgs a) {
     __shared__ double vprev[kLzSmallN], vcur[kLzSmallN], w[kLzSmallN];
     __shared__ __align__(16) float v32[kLzSmallN];
-    __shared__ double sh[kLzSmallThreads / 32 + 1];
+    __shared__ double sh[2][kLzVecThreads / 32], norm[2];
+    __shared__ bool done;
     __shared__ int item;
     extern __shared__ float4 hcache4[];             // rows 0 .. rc - 1 of H (FP32), pitch pc
     float* const hcache = reinterpret_cast<float*>(hcache4);
@@ -245,17 +287,24 @@ __global__ void __launch_bounds__(kLzSmallThreads, 1) lanczos_small_kernel(Lancz
             hcache[i] = c < n ? Hb[(size_t)r * a.P + c] : 0.f;
         }
         // v_1 from the counter-based generator, v_0 = 0
-        double s = 0.0;
-        for (int i = t; i < n; i += kLzSmallThreads) {
-            const double q = 2.0 * ((double)(splitmix64((unsigned long long)i) >> 11) * 0x1.0p-53) - 1.0;
-            vcur[i] = q;
-            vprev[i] = 0.0;
-            s += q * q;
-        }
-        const double nrm = sqrt(block_sum<kLzSmallThreads>(s, sh));
-        for (int i = t; i < n; i += kLzSmallThreads) {
-            vcur[i] /= nrm;
-            v32[i] = (float)vcur[i];
+        if (t < kLzVecThreads) {
+            double s = 0.0;
+            for (int i = t; i < n; i += kLzVecThreads) {
+                const double q = 2.0 * ((double)(splitmix64((unsigned long long)i) >> 11) * 0x1.0p-53) - 1.0;
+                vcur[i] = q;
+                vprev[i] = 0.0;
+                s += q * q;
+            }
+            s = vec_sum(s, sh[1]);
+            if (t == 0) {
+                norm[0] = sqrt(s);
+                norm[1] = 1.0 / norm[0];
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(kLzVecThreads) : "memory");
+            for (int i = t; i < n; i += kLzVecThreads) {
+                vcur[i] = div_by(vcur[i], norm[0], norm[1]);
+                v32[i] = (float)vcur[i];
+            }
         }
         __syncthreads();
         double* ab = a.ab + (size_t)b * kLzSteps * 2;
@@ -304,36 +353,44 @@ __global__ void __launch_bounds__(kLzSmallThreads, 1) lanczos_small_kernel(Lancz
                 }
             }
             __syncthreads();
-            double p = 0.0;
-            for (int i = t; i < n; i += kLzSmallThreads) p += w[i] * vcur[i];
-            const double alpha = block_sum<kLzSmallThreads>(p, sh);
-            p = 0.0;
-            for (int i = t; i < n; i += kLzSmallThreads) {
-                const double wi = w[i] - alpha * vcur[i];
-                w[i] = wi;
-                p += wi * wi;
-            }
-            const double beta = sqrt(block_sum<kLzSmallThreads>(p, sh));
-            if (j == 0) {
-                a1 = alpha;
-                b1 = beta;
-            }
-            if (t == 0) {
-                ab[2 * j] = alpha;
-                ab[2 * j + 1] = beta;
-            }
-            m = j + 1;
-            stop = beta <= 1e-12 * (fabs(a1) + b1 + 1.0);      // the same on every thread
-            if (!stop) {
-                for (int i = t; i < n; i += kLzSmallThreads) {
-                    const double v = w[i] / beta;
-                    vprev[i] = vcur[i];
-                    vcur[i] = v;
-                    v32[i] = (float)v;
+            if (t < kLzVecThreads) {
+                double p = 0.0;
+                for (int i = t; i < n; i += kLzVecThreads) p += w[i] * vcur[i];
+                const double alpha = vec_sum(p, sh[0]);
+                p = 0.0;
+                for (int i = t; i < n; i += kLzVecThreads) {
+                    const double wi = w[i] - alpha * vcur[i];
+                    w[i] = wi;
+                    p += wi * wi;
                 }
-                bprev = beta;
+                p = vec_sum(p, sh[1]);
+                if (t == 0) {
+                    const double beta = sqrt(p);
+                    if (j == 0) {
+                        a1 = alpha;
+                        b1 = beta;
+                    }
+                    ab[2 * j] = alpha;
+                    ab[2 * j + 1] = beta;
+                    norm[0] = beta;
+                    norm[1] = 1.0 / beta;
+                    done = beta <= 1e-12 * (fabs(a1) + b1 + 1.0);
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(kLzVecThreads) : "memory");
+                if (!done) {
+                    const double beta = norm[0], rbeta = norm[1];
+                    for (int i = t; i < n; i += kLzVecThreads) {
+                        const double v = div_by(w[i], beta, rbeta);
+                        vprev[i] = vcur[i];
+                        vcur[i] = v;
+                        v32[i] = (float)v;
+                    }
+                }
             }
             __syncthreads();
+            m = j + 1;
+            stop = done;
+            bprev = norm[0];
         }
         if (t == 0) a.state[b] = m | (stop ? kLzStopped : 0);
         __syncthreads();
