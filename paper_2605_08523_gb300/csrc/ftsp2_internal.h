@@ -327,6 +327,32 @@ cudaError_t launch_train_absmax(const double* dR, int ns, double* dPart, double*
 
 void count_launch(int n = 1);
 
+// Launch that may be prepared while the kernel before it in the stream still runs
+// (programmatic stream serialisation).  Every kernel launched so begins, in every
+// thread and before it reads or writes memory or returns, with grid_wait(), which
+// ends when the kernel before it has completed and its writes are visible.  A
+// kernel whose successor may take its place on the SMs early calls
+// grid_trigger() after that: the one-block and setup kernels, not those whose
+// successor's CTAs would then be packed onto the SMs that finish first.
+// Cooperative launches are ordinary ones.  n = 256 (seven kernels, 1 to 3 us
+// between two of them before): 265 -> 252 us; mu search at 512 (29 kernels): 1440
+// -> 1388; n = 1728 with 24 Lanczos steps (68 kernels): 3393 -> 3246.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // --- inputs of the training built by the library (train_inputs.cu, host) ----------
 // N sample points of [0, 1] at the quantiles of p = 1 + |f'| (seed 0: cell
 // midpoints; else splitmix64-drawn positions inside the N cells)
@@ -388,6 +414,9 @@ __device__ __forceinline__ unsigned long long globaltimer() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

@@ -79,6 +79,8 @@ __device__ __forceinline__ double* lz_vec(const LanczosArgs& a, int which, int b
 
 // v_1 from the counter-based generator; v_0 = 0; steps done = 0
 __global__ void __launch_bounds__(kLzThreads) lanczos_start_kernel(LanczosArgs a) {
+    grid_wait();
+    grid_trigger();
     __shared__ double sh[kLzThreads / 32 + 1];
     const int b = blockIdx.x;
     const int n = a.inst[b].n;
@@ -114,6 +116,8 @@ __device__ __forceinline__ bool lz_active(const LanczosArgs& a, int b, int j, in
 // w = H v_j - beta_{j-1} v_{j-1}; per block (kLzRows rows, one warp each) the
 // partial sum of w . v_j
 __global__ void __launch_bounds__(kLzRows * 32) lanczos_matvec_kernel(LanczosArgs a, int j) {
+    grid_wait();
+    grid_trigger();
     const int b = blockIdx.y;
     const int n = a.inst[b].n;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -155,6 +159,8 @@ __global__ void __launch_bounds__(kLzRows * 32) lanczos_matvec_kernel(LanczosArg
 // alpha_j, w -= alpha_j v_j, beta_j = ||w||, v_{j+1} = w / beta_j (into the
 // buffer of v_{j-1}); one block per instance
 __global__ void __launch_bounds__(kLzThreads) lanczos_update_kernel(LanczosArgs a, int j) {
+    grid_wait();
+    grid_trigger();
     __shared__ double sh[kLzThreads / 32 + 1];
     const int b = blockIdx.x;
     const int n = a.inst[b].n;
@@ -232,6 +238,8 @@ constexpr int kLzSortMax = 8192;
 __device__ __forceinline__ int* lz_queue(const LanczosArgs& a) { return reinterpret_cast<int*>(a.part); }
 
 __global__ void lanczos_queue_kernel(LanczosArgs a) {
+    grid_wait();
+    grid_trigger();
     int* const queue = lz_queue(a);
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b == 0) queue[0] = 0;
@@ -261,6 +269,7 @@ __device__ __forceinline__ double vec_sum(double v, double* sh) {
 }
 
 __global__ void __launch_bounds__(kLzSmallThreads, 1) lanczos_small_kernel(LanczosArgs a) {
+    grid_wait();
     __shared__ double vprev[kLzSmallN], vcur[kLzSmallN], w[kLzSmallN];
     __shared__ __align__(16) float v32[kLzSmallN];
     __shared__ double sh[2][kLzVecThreads / 32], norm[2];
@@ -473,6 +482,8 @@ __device__ __forceinline__ double edge_vector_last(const double* al, const doubl
 // operations; one instance took 379 us with one warp, divisions in the Sturm
 // counts and the factors formed anew in each solve, 84 us now.
 __global__ void __launch_bounds__(64) lanczos_bounds_kernel(LanczosArgs a) {
+    grid_wait();
+    grid_trigger();
     __shared__ double al[kLzSteps], be[kLzSteps], sal[kLzSteps], sb2[kLzSteps];
     __shared__ double edge[2], res[2];
     const int lane = threadIdx.x & 31, upper = threadIdx.x >> 5;
@@ -582,22 +593,23 @@ void launch_lanczos(const LanczosArgs& a, int max_n, int sms, cudaStream_t s) {
                                  kLzSmallCacheBytes);
             attr = true;
         }
-        lanczos_queue_kernel<<<(a.nb + 255) / 256, 256, 0, s>>>(a);
-        lanczos_small_kernel<<<std::min(a.nb, std::max(1, sms)), kLzSmallThreads, kLzSmallCacheBytes, s>>>(a);
-        lanczos_bounds_kernel<<<a.nb, 64, 0, s>>>(a);
+        launch_after(lanczos_queue_kernel, dim3((a.nb + 255) / 256), dim3(256), 0, s, a);
+        launch_after(lanczos_small_kernel, dim3(std::min(a.nb, std::max(1, sms))), dim3(kLzSmallThreads),
+                     kLzSmallCacheBytes, s, a);
+        launch_after(lanczos_bounds_kernel, dim3(a.nb), dim3(64), 0, s, a);
         count_launch(3);
         return;
     }
-    lanczos_start_kernel<<<a.nb, kLzThreads, 0, s>>>(a);
+    launch_after(lanczos_start_kernel, dim3(a.nb), dim3(kLzThreads), 0, s, a);
     count_launch();
     const int steps = max_n < kLzSteps ? max_n : kLzSteps;
     const dim3 mgrid((max_n + kLzRows - 1) / kLzRows, a.nb);
     for (int j = 0; j < steps; ++j) {
-        lanczos_matvec_kernel<<<mgrid, kLzRows * 32, 0, s>>>(a, j);
-        lanczos_update_kernel<<<a.nb, kLzThreads, 0, s>>>(a, j);
+        launch_after(lanczos_matvec_kernel, mgrid, dim3(kLzRows * 32), 0, s, a, j);
+        launch_after(lanczos_update_kernel, dim3(a.nb), dim3(kLzThreads), 0, s, a, j);
         count_launch(2);
     }
-    lanczos_bounds_kernel<<<a.nb, 64, 0, s>>>(a);
+    launch_after(lanczos_bounds_kernel, dim3(a.nb), dim3(64), 0, s, a);
     count_launch();
 }
 

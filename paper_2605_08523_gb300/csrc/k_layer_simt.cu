@@ -49,6 +49,7 @@ __device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float((unsigned
 
 __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_constant__ LayerArgs a) {
     __shared__ __align__(16) float sm[kSStages * 2 * kSK * kSQ];
+    grid_wait();
     // no instance starts before status[1]: a layer below it has nothing to do
     if (a.gl < *reinterpret_cast<volatile const int*>(a.status + 1)) return;
     const int t = blockIdx.x >> 2, quad = blockIdx.x & 3;
@@ -169,9 +170,9 @@ __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_c
 }
 
 cudaError_t launch_layer_simt(const LayerArgs& a, cudaStream_t s) {
-    layer_simt_kernel<<<4 * a.ntiles, kSThreads, 0, s>>>(a);
+    const cudaError_t e = launch_after(layer_simt_kernel, dim3(4 * a.ntiles), dim3(kSThreads), 0, s, a);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ftsp2

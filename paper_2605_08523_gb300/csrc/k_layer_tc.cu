@@ -1004,6 +1004,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
     // A launch whose layers all lie below the first layer any instance starts
     // at (models with fewer layers than the set's maximum start late) has no
     // active item: every thread of both CTAs of a pair leaves at once.
+    grid_wait();
     const int first_layer = *reinterpret_cast<volatile const int*>(a.status + 1);
     if (a.gl + a.nlayers <= first_layer) return;
     extern __shared__ uint8_t smem_raw[];
@@ -1568,6 +1569,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
     // A launch whose layers all lie below the first layer any instance starts
     // at (models with fewer layers than the set's maximum start late) has no
     // active item: every thread of both CTAs of a pair leaves at once.
+    grid_wait();
     const int first_layer = *reinterpret_cast<volatile const int*>(a.status + 1);
     if (a.gl + a.nlayers <= first_layer) return;
     // the items of layers before the first active one are skipped by every role
@@ -2117,8 +2119,11 @@ struct Variant {
         if (a.nlayers > 1) {
             attr[cfg.numAttrs].id = cudaLaunchAttributeCooperative;
             attr[cfg.numAttrs].val.cooperative = 1;
-            ++cfg.numAttrs;
+        } else {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         }
+        ++cfg.numAttrs;
         e = cudaLaunchKernelEx(&cfg, fn(), a, *m.rd[0], *m.rd[1], *m.wr[0], *m.wr[1]);
         count_launch();
         return e;

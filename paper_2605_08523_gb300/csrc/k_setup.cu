@@ -100,6 +100,8 @@ __device__ __forceinline__ void write_tiles(const ftsp2_instance* inst, int nb, 
 // long-K tiles are dealt first and every unit's last tiles are short ones.  All
 // tiles of chain 0, then those of chain 1.
 __global__ void __launch_bounds__(kPrepThreads) prep_kernel(SetupArgs a) {
+    grid_wait();
+    grid_trigger();
     __shared__ int ns[kTileSortMax], order[kTileSortMax], pre[kTileSortMax + 1];
     const int t = threadIdx.x;
     for (int b = t; b < a.nb; b += kPrepThreads) {
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(SetupArgs a) {
 }
 
 void launch_prep(const SetupArgs& a, cudaStream_t s) {
-    prep_kernel<<<1, kPrepThreads, 0, s>>>(a);
+    launch_after(prep_kernel, dim3(1), dim3(kPrepThreads), 0, s, a);
     count_launch();
 }
 
@@ -195,6 +197,8 @@ void launch_prep(const SetupArgs& a, cudaStream_t s) {
 constexpr int kGWarps = 8;
 
 __global__ void __launch_bounds__(kGWarps * 32) gershgorin_kernel(SetupArgs a) {
+    grid_wait();
+    grid_trigger();
     const int b = blockIdx.y;
     const int n = a.inst[b].n;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(kGWarps * 32) gershgorin_kernel(SetupArgs a) {
 
 void launch_gershgorin(const SetupArgs& a, int max_n, cudaStream_t s) {
     dim3 grid((max_n + kGWarps - 1) / kGWarps, a.nb);
-    gershgorin_kernel<<<grid, kGWarps * 32, 0, s>>>(a);
+    launch_after(gershgorin_kernel, grid, dim3(kGWarps * 32), 0, s, a);
     count_launch();
 }
 
@@ -312,6 +316,8 @@ __device__ __forceinline__ int pick_model(const SetupArgs& a, bool min_layers, i
 // model's region took most of the time when one thread walked the set: 12 us for
 // the twelve models of the ragged set, 6 us now).
 __global__ void decide_kernel(SetupArgs a) {
+    grid_wait();
+    grid_trigger();
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= a.nb) return;
     const ftsp2_instance in = a.inst[b];
@@ -408,7 +414,7 @@ __global__ void decide_kernel(SetupArgs a) {
 }
 
 void launch_decide(const SetupArgs& a, cudaStream_t s) {
-    decide_kernel<<<(a.nb + 3) / 4, 128, 0, s>>>(a);
+    launch_after(decide_kernel, dim3((a.nb + 3) / 4), dim3(128), 0, s, a);
     count_launch();
 }
 
@@ -516,6 +522,7 @@ __device__ __forceinline__ void write_operand16(int fmt, uint8_t* base, size_t p
 // (-scale) * H_rc elsewhere (the same value as scale * (0 - H_rc)).
 
 __global__ void __launch_bounds__(256) init_kernel(InitArgs a) {
+    grid_wait();
     const int b = blockIdx.y;
     const ftsp2_instance in = a.inst[b];
     const int n = in.n, P = a.P;
@@ -643,7 +650,7 @@ void launch_init(const InitArgs& a, int max_n, cudaStream_t s) {
     InitArgs args = a;
     args.cols = (size_t)a.nb * a.P * a.P >= (size_t)1536 * 1536 ? 512 : 128;
     dim3 grid((a.P + 31) / 32, a.nb, (a.P + args.cols - 1) / args.cols);
-    init_kernel<<<grid, 256, 0, s>>>(args);
+    launch_after(init_kernel, dim3(grid), dim3(256), 0, s, args);
     count_launch();
 }
 
@@ -664,6 +671,7 @@ void launch_init(const InitArgs& a, int max_n, cudaStream_t s) {
 constexpr int kFinThreads = 256;
 
 __global__ void __launch_bounds__(kMaxChains * kFinThreads) finalize_kernel(FinalArgs a) {
+    grid_wait();
     const int b = blockIdx.x;
     __shared__ double s_sum[kMaxChains][kFinThreads / 32][2];
     __shared__ int s_bad[kMaxChains];
@@ -750,6 +758,8 @@ __global__ void __launch_bounds__(kMaxChains * kFinThreads) finalize_kernel(Fina
 // valid model.  One thread per instance.
 // ------------------------------------------------------------------------------
 __global__ void mu_update_kernel(MuArgs a) {
+    grid_wait();
+    grid_trigger();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= a.nb) return;
     const ftsp2_rescale_rec rec = a.rec[b];
@@ -767,12 +777,12 @@ __global__ void mu_update_kernel(MuArgs a) {
 }
 
 void launch_mu_update(const MuArgs& a, cudaStream_t s) {
-    mu_update_kernel<<<(a.nb + 127) / 128, 128, 0, s>>>(a);
+    launch_after(mu_update_kernel, dim3((a.nb + 127) / 128), dim3(128), 0, s, a);
     count_launch();
 }
 
 void launch_finalize(const FinalArgs& a, cudaStream_t s) {
-    finalize_kernel<<<a.nb, a.nchains * kFinThreads, 0, s>>>(a);
+    launch_after(finalize_kernel, dim3(a.nb), dim3(a.nchains * kFinThreads), 0, s, a);
     count_launch();
 }
 
