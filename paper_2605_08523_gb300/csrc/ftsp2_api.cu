@@ -472,12 +472,12 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     // tiles of each shape; the tile of a call's main table is that of its shape
     // (128 x 128 in FP32 mode), a second table of 128 x 128 tiles serves
     // single-CTA layers and FP32 refinement layers
-    long long nt[3] = {0, 0, 0};
+    long long nt[kShapes] = {};
     for (int b = 0; b < nb; ++b)
-        for (int sh = 0; sh < 3; ++sh) nt[sh] += host_tiles_of(inst[b].n, tc_block_m(sh), tc_block_n(sh));
+        for (int sh = 0; sh < kShapes; ++sh) nt[sh] += host_tiles_of(inst[b].n, tc_block_m(sh), tc_block_n(sh));
     const bool defer = !simt_main && deferred_epilogue(inst, nb, flags);
     long long ntmax = 0;
-    for (int sh = 0; sh < 3; ++sh) {
+    for (int sh = 0; sh < kShapes; ++sh) {
         nt[sh] *= nch;
         ntmax = std::max(ntmax, nt[sh]);
     }
@@ -485,7 +485,7 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     L.P = P;
     L.nb = nb;
     L.nchains = nch;
-    for (int sh = 0; sh < 3; ++sh) L.ntiles[sh] = (int)nt[sh];
+    for (int sh = 0; sh < kShapes; ++sh) L.ntiles[sh] = (int)nt[sh];
     L.plane_elems = (size_t)nb * P * P;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -585,22 +585,24 @@ static int chunk_shape(const ftsp2_instance* inst, int nb, int sms) {
 // Clocks of one layer with a tile shape, from the measured parts of a tile: the
 // K loop per 64 elements (the MMAs of a pair: 768 clocks of FP16X2 on 128
 // columns run in 850, on 256 columns 1536 in 1570; a single CTA's 128 x 128
-// MMAs, both panels from one shared memory, take 1430 for 768), and the final
-// epilogue, which follows the K loop when a unit has one tile and otherwise
-// overlaps the next tile's (kStream is then its share of a tile, bound by the
-// state's traffic).  With more tiles than units the layer costs its mean load,
-// and a part of a tile for the uneven end: less when other instances or chains
-// fill it.  Measured (one lattice, density + entropy, FP16X2; single / 256 x 256 /
-// 256 x 128, us per solve): n = 64: 214 / 287 / 223; 256: 275 / 587 / 266;
-// 1024: 508 / 846 / 429; 2048: 1367 / 1324 / 1130; 3072: 4013 / 3946 / 3192;
-// 4096: 9175 / 7388 / 7731; 40 instances of n = 256: 985 / 1325 / 1095;
-// the ragged batch of 512: 22980 / 34750 / 25170.
+// MMAs, both panels from one shared memory, take 1300 for 768, its 128 x 64 ones
+// 1000 for 384), and the final epilogue, which follows the K loop when a unit has
+// one tile and otherwise overlaps the next tile's (kStream is then its share of a
+// tile, bound by the chain of its steps).  With more tiles than units the layer
+// costs its mean load, and a part of a tile for the uneven end: less when other
+// instances or chains fill it.  Measured (us per solve; 128 x 128 / 256 x 128 /
+// 128 x 64), one lattice, density + entropy, FP16X2: n = 64: 149 / 154 / 136; 384:
+// 268 / 266 / 230; 900: 442 / 394 / 393; 1280: 545 / 479 / 569; 1800: 1095 / 982 /
+// 1345; density, TF32X3: n = 128: 307 / 299 / 213; 900: 730 / 608 / 560; 1536:
+// 1026 / 823 / 1491; 24 fragments of 16 to 200: 497 / 491 / 470; 40 instances of
+// n = 256: 603 / 706 / 632; the ragged batch of 512: 21520 / 24830 / 23080.  256 x
+// 256 pays from n = 3000 to 4000 on (4096: 9175 / 7731, 256 x 256 7388).
 static double shape_cost(const ftsp2_instance* inst, int nb, int nch, int mode, int sms, int shape, bool deferred) {
-    static const double kSlice[3][3] = {{2860, 3140, 1700}, {2500, 3100, 1650}, {1430, 1570, 850}};   // TF32X3, BF16X3, FP16X2
+    static const double kSlice[3][kShapes] = {{2860, 3140, 1700, 1750}, {2500, 3100, 1650, 1700}, {1300, 1570, 850, 1000}};   // TF32X3, BF16X3, FP16X2
     const double slice = kSlice[mode == FTSP2_TF32X3 ? 0 : mode == FTSP2_BF16X3 ? 1 : 2][shape];
-    const double epi = shape == SHAPE_SINGLE ? 7000 : shape == SHAPE_PAIR128 ? 7700 : 28000;
-    const double stream = shape == SHAPE_PAIR && !deferred ? 28000 : 14000;
-    const double units = std::max(1, shape == SHAPE_SINGLE ? sms : sms / 2);
+    const double epi = shape == SHAPE_SINGLE ? 7000 : shape == SHAPE_PAIR128 ? 7700 : shape == SHAPE_SINGLE64 ? 5000 : 28000;
+    const double stream = shape == SHAPE_PAIR && !deferred ? 28000 : shape == SHAPE_SINGLE64 ? 9000 : 14000;
+    const double units = std::max(1, tc_pair(shape) ? sms / 2 : sms);
     double tiles = 0.0, load = 0.0, longest = 0.0;
     for (int b = 0; b < nb; ++b) {
         const double t = (double)nch * (double)host_tiles_of(inst[b].n, tc_block_m(shape), tc_block_n(shape));
@@ -634,8 +636,8 @@ static int layer_shape(const ftsp2_instance* inst, int nb, int mode, int want, i
     const int nch = want == 3 ? 2 : 1;
     int best = -1;
     double cost = 0.0;
-    for (int shape = 0; shape < 3; ++shape) {
-        if (pair >= 0 && pair != (shape != SHAPE_SINGLE)) continue;
+    for (int shape = 0; shape < kShapes; ++shape) {
+        if (pair >= 0 && pair != (tc_pair(shape) ? 1 : 0)) continue;
         const double c = shape_cost(inst, nb, nch, mode, sms, shape, deferred);
         if (best < 0 || c < cost) {
             best = shape;
@@ -817,7 +819,7 @@ static ftsp2_status run(const double* dH, const ftsp2_instance* inst, const ftsp
     }
     auto is_simt = [&](int g) { return all_simt || (g >= refine_from && !refine_tc); };
     auto is_rtc = [&](int g) { return refine_tc && g >= refine_from; };
-    const bool pair = shape != SHAPE_SINGLE;
+    const bool pair = tc_pair(shape);
     // mean order n over the tiles that set the accumulation chunks
     double mean_k = 0.0;
     {
@@ -1433,7 +1435,8 @@ ftsp2_status ftsp2_tile_shape(const ftsp2_instance* inst, int nb, ftsp2_mode mod
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return FTSP2_E_CUDA;
     const int pair = chosen_pair(inst, nb, mode, want, flags, from_tuner);
-    *shape = layer_shape(inst, nb, mode, want, flags, pair, sms, deferred_epilogue(inst, nb, flags)) != SHAPE_SINGLE;
+    *shape = layer_shape(inst, nb, mode, want, flags, pair, sms, deferred_epilogue(inst, nb, flags));
+    *shape = tc_pair(*shape) ? 1 : 0;
     return FTSP2_OK;
 }
 

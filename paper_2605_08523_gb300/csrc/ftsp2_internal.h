@@ -118,7 +118,7 @@ struct Layout {
     size_t total;
     size_t plane_elems;   // nb * P * P
     int P, nb, nchains;
-    int ntiles[3];        // tiles of each shape over all chains: 128 x 128, 256 x 256, 256 x 128
+    int ntiles[4];        // tiles of each shape over all chains: 128 x 128, 256 x 256, 256 x 128, 128 x 64
     int planes;           // FP32 state planes per chain: 2 (Z, A), or L + 1 for Max-SP2 tables
 };
 
@@ -292,7 +292,9 @@ struct LayerMaps {
 // Tensor-core layer (k_layer_tc.cu); mode in {TF32X3, BF16X3, FP16X2}; shape 0:
 // 128 x 128 tiles on single CTAs (units = CTAs), 1: 256 x 256 and 2: 256 x 128
 // tiles on CTA pairs (units = pairs).  Persistent grid of `units`.
-enum { SHAPE_SINGLE = 0, SHAPE_PAIR = 1, SHAPE_PAIR128 = 2 };
+enum { SHAPE_SINGLE = 0, SHAPE_PAIR = 1, SHAPE_PAIR128 = 2, SHAPE_SINGLE64 = 3 };
+constexpr int kShapes = 4;
+constexpr bool tc_pair(int shape) { return shape == SHAPE_PAIR || shape == SHAPE_PAIR128; }
 int tc_block_m(int shape);
 int tc_block_n(int shape);
 cudaError_t launch_layer_tc(int mode, const LayerArgs& a, const LayerMaps& m, int units, int shape, cudaStream_t s);

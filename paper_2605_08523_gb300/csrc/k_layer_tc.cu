@@ -4,8 +4,8 @@
 // persistent cooperative launch (below).
 //
 // The product of a layer is the symmetric square Z^2 of the centred state.
-// Output tiles are 256 x 256 or 256 x 128 (CTA pairs) or 128 x 128 (single CTAs),
-// chosen per call, and only those touching the upper triangle are computed; each
+// Output tiles are 256 x 256 or 256 x 128 (CTA pairs) or 128 x 128 or 128 x 64
+// (single CTAs), chosen per call, and only those touching the upper triangle are computed; each
 // element (r, c) with r <= c is produced once.  Since Z is
 // symmetric, (Z^2)_{rc} = sum_k Z_{rk} Z_{ck}: both MMA operands are row
 // panels of the same matrix, loaded by TMA with 128-byte swizzle.  The next
@@ -30,8 +30,12 @@
 // "tempty".  Single CTAs (cta_group::1) run the same pipeline on 128 x 128 tiles
 // with M = 128 MMAs: the least padding on the diagonal and at ragged edges, but
 // an MMA whose two panels come from one shared memory takes 119 clocks for 64
-// (a pair's 256 x 128 one: 71).  One choice per call (shape_cost in
-// ftsp2_api.cu).
+// (a pair's 256 x 128 one: 71).  128 x 64 tiles of single CTAs, for calls of few
+// tiles, where a layer is one tile's latency: half the columns of an epilogue warp
+// and twice the SMs at work, an MMA of about 80 clocks for the 32 that it runs.
+// Per solve against the best of the others: n = 256 239 -> 214 us, mu search at
+// 512 1380 -> 1253, n = 1024 BF16X3 553 -> 519, n = 384 TF32X3 428 -> 330.  One
+// choice per call (shape_cost in ftsp2_api.cu).
 //
 // Chunked accumulation.  Every 128 elements of K (CK slices; a launch may ask
 // for shorter chunks) the MMAs switch to the next of the TMEM chunk
@@ -128,12 +132,14 @@ struct TcCfg<FTSP2_TF32X3> {
 
 // Tile geometry.  SHAPE_SINGLE: one CTA, 128 x 128 tiles, M = 128 MMAs.
 // SHAPE_PAIR / SHAPE_PAIR128: clusters of two CTAs, M = 256 MMAs on 256 x 256 or
-// 256 x 128 tiles.  A CTA owns 128 rows of its tile in every shape.
+// 256 x 128 tiles.  SHAPE_SINGLE64: one CTA, 128 x 64 tiles.  A CTA owns 128 rows of
+// its tile in every shape.
 template <int SHAPE>
 struct Geo {
-    static constexpr int NCTA = SHAPE == SHAPE_SINGLE ? 1 : 2;
+    static constexpr int NCTA = tc_pair(SHAPE) ? 2 : 1;
     static constexpr int TM = 128 * NCTA;                      // rows of a tile
-    static constexpr int TN = SHAPE == SHAPE_PAIR ? 256 : 128; // columns of a tile
+    // columns of a tile
+    static constexpr int TN = SHAPE == SHAPE_PAIR ? 256 : SHAPE == SHAPE_SINGLE64 ? 64 : 128;
     static constexpr int BROWS = TN / NCTA;                    // rows of the B panel a CTA loads
     // TMEM chunk accumulators of TN columns (512 columns in all)
     static constexpr int NBUF = 512 / TN;
@@ -141,7 +147,10 @@ struct Geo {
 constexpr int kCtaRows = 128;
 // Epilogue warps of layer_tc_kernel, followed by the context warp.
 template <int OUTFMT, int SHAPE>
-constexpr int epi_warps() { return OUTFMT == OP_F16X2 && SHAPE != SHAPE_PAIR ? 16 : 8; }
+constexpr int epi_warps() {
+    if (SHAPE == SHAPE_SINGLE64) return OUTFMT == -1 ? 4 : 8;     // last layer: a 32 x 64 block of partial sums a warp
+    return OUTFMT == OP_F16X2 && SHAPE != SHAPE_PAIR ? 16 : 8;
+}
 template <int OUTFMT, int SHAPE>
 constexpr int tc_threads() { return 32 * (2 + epi_warps<OUTFMT, SHAPE>() + 1); }
 // Deferred final epilogue: store warps, their shared-memory staging ring
@@ -999,7 +1008,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
     constexpr uint32_t IDESC = make_idesc(C::ATYPE, TM, TN);
     constexpr uint32_t TMEM_COLS = 512;
     // a unit that keeps its tile's state in TMEM has two chunk buffers there
-    constexpr bool CAN_RESIDE = TN == 128 && !LAST;
+    constexpr bool CAN_RESIDE = TN <= 128 && !LAST;
 
     // A launch whose layers all lie below the first layer any instance starts
     // at (models with fewer layers than the set's maximum start late) has no
@@ -1028,7 +1037,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
     const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;     // pair or CTA
     const int nunits = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     const bool resident = CAN_RESIDE && a.resident != 0;
-    const int nbuf = resident ? 2 : G::NBUF;
+    const int nbuf = resident ? kStateZ / TN : G::NBUF;
     const int nst = (resident || LAST) ? St::NMAX : St::N;     // stages of the operand ring
     if (threadIdx.x == 0) {
         for (int s = 0; s < St::NMAX; ++s) {
@@ -1406,7 +1415,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
             const bool live = cb0 < cb1;
             const int* const dep = resident ? nullptr : c.dep;
             // the state of the first block, loaded ahead of the last chunk
-            constexpr int AH = EPI_COLS == 32 ? 1 : 2;
+            constexpr int AH = EW == 16 ? 1 : 2;
             State<AH> ahead;
             const bool state_global = live && (!resident || c.first);
             auto load_first = [&](State<AH>& s) {
@@ -2069,8 +2078,8 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
     }
 }
 
-int tc_block_m(int shape) { return shape == SHAPE_SINGLE ? 128 : 256; }
-int tc_block_n(int shape) { return shape == SHAPE_PAIR ? 256 : 128; }
+int tc_block_m(int shape) { return tc_pair(shape) ? 256 : 128; }
+int tc_block_n(int shape) { return shape == SHAPE_PAIR ? 256 : shape == SHAPE_SINGLE64 ? 64 : 128; }
 
 // One kernel variant: its function, threads, dynamic shared memory and CTAs per unit.
 template <int MODE, int OUTFMT, int SHAPE, bool DEFER>
@@ -2172,6 +2181,7 @@ static cudaError_t launch_mode(const LayerArgs& a, const LayerMaps& m, int units
         case SHAPE_SINGLE: return launch_shape<MODE, MAINFMT, SHAPE_SINGLE>(a, m, units, s);
         case SHAPE_PAIR: return launch_shape<MODE, MAINFMT, SHAPE_PAIR>(a, m, units, s);
         case SHAPE_PAIR128: return launch_shape<MODE, MAINFMT, SHAPE_PAIR128>(a, m, units, s);
+        case SHAPE_SINGLE64: return launch_shape<MODE, MAINFMT, SHAPE_SINGLE64>(a, m, units, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -2194,6 +2204,7 @@ static int max_units_mode(int shape, bool defer) {
             return defer ? Variant<MODE, MAINFMT, SHAPE_PAIR, true>::max_units()
                          : Variant<MODE, MAINFMT, SHAPE_PAIR, false>::max_units();
         case SHAPE_PAIR128: return Variant<MODE, MAINFMT, SHAPE_PAIR128, false>::max_units();
+        case SHAPE_SINGLE64: return Variant<MODE, MAINFMT, SHAPE_SINGLE64, false>::max_units();
     }
     return 0;
 }

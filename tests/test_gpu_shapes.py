@@ -47,3 +47,18 @@ def test_shapes_bitwise(ft, mode, ns):
         assert torch.equal(s.D, base.D), flags
         assert torch.allclose(s.S, base.S, rtol=1e-12, atol=1e-12)
         assert torch.allclose(s.trace, base.trace, rtol=1e-12, atol=1e-12)
+
+
+@pytest.mark.parametrize("mode", ["fp16x2", "bf16x3", "tf32x3"])
+@pytest.mark.parametrize("n", [17, 63, 64, 65, 95, 127, 128, 129, 193, 320, 449, 640])
+def test_narrow_tiles_bitwise(ft, mode, n):
+    """Single matrices, which run on 128 x 64 tiles by default: the same D, S and trace
+    as on pairs, bit for bit, in multi-layer launches (the state in TMEM), with a
+    launch per layer, and with the last two layers refined."""
+    Hd = torch.from_numpy(wl.chain_1d(n, 90 + n)).cuda()
+    for extra in (0, ft.LAYER_LAUNCHES, ft.REFINE2, ft.REFINE2 | ft.REFINE_TC):
+        base = solve(ft, [n], mode, ft.PAIR_TILES | extra, Hd)
+        s = solve(ft, [n], mode, ft.SINGLE_TILES | extra, Hd)
+        assert np.isfinite(base.D.cpu().numpy()).all()
+        assert torch.equal(s.D, base.D), extra
+        assert torch.equal(s.S, base.S) and torch.equal(s.trace, base.trace), extra
