@@ -67,6 +67,22 @@ def test_one_lm_step_matches_oracle(ft, seed):
     assert abs(rep["cost"] - hist[0][0]) < 1e-9 * hist[0][0]
 
 
+@pytest.mark.parametrize("L, ns", [(3, 255), (3, 257), (12, 256), (16, 2000), (45, 300), (46, 300), (47, 700),
+                                   (48, 1021), (64, 257)])
+def test_one_accelerated_step_matches_oracle(ft, L, ns):
+    # the right-hand side of the second solve at the edges of the 256-sample blocks
+    # and on either side of the width up to which slices hold 16 samples.  Damping
+    # 1e-3 of the diagonal bounds the scaled condition number by 4 L / 1e-3 = 2e5;
+    # the second difference at h = 0.1 multiplies rounding by 200: 2e5 x 200 x 1e-16
+    # of the correction, held to 1e-6 of the table.
+    beta0, mu0 = 40.0, 1 / 3
+    x = train.sample_grid(ns, beta0, mu0, seed=1)
+    th0 = train.init_from_sp2(L, beta0, mu0)
+    th_or, _ = train.lm_fit(th0, x, beta0=beta0, mu0=mu0, iters=1, accel=True)
+    th_gpu, _ = ft.ftsp2_train_coeffs(ft.TARGET_FERMI, beta0, mu0, L=L, nsamples=ns, seed=1, iterations=1, accel=True)
+    assert np.max(np.abs(th_gpu - th_or)) < 1e-6 * max(1.0, np.max(np.abs(th_or)))
+
+
 def test_training_gain_over_sp2(ft):
     # beta0 = 40, mu0 = 1/3, 12 layers: the SP2-mu table misses the Fermi
     # function by ~0.3; LM with geodesic acceleration on the GPU brings the
