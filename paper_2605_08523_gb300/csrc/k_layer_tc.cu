@@ -70,8 +70,9 @@
 // last buffer, which stays held.  Where a launch has one tile per unit, Z and A
 // of that tile stay in TMEM from layer to layer.
 // One lattice, density + entropy, FP16X2, per solve, before (single CTAs, 576
-// threads) and after: n = 256: 402 -> 285 us (with the rest of a solve); n =
-// 1501 (entropy): 789 -> 516 us; n = 1024 BF16X3 (density): 812 -> 580 us.
+// threads, operands written by plain stores) and now, the rest of a solve
+// included: n = 256: 402 -> 208 us; n = 1501 (entropy): 789 -> 498 us; n = 1024
+// BF16X3 (density): 814 -> 520 us; n = 2048 TF32X3 (density): 2567 -> 2208 us.
 //
 // layer_defer_kernel (640 threads; 256 x 256 tiles with long K).  Sixteen
 // accumulating warps store a tile's sums to a per-CTA scratch in global memory
