@@ -560,6 +560,11 @@ def table_paths(args):
     return paths
 
 
+def tile_label(solver, shape):
+    """Size and kind of the tiles that the solver runs on (shape: 1 pair, 0 single, -1 none)."""
+    return "none" if shape < 0 else "%dx%d %s" % (*solver.tile_size(), "CTA pairs" if shape else "single CTAs")
+
+
 def flags_of(args, ft):
     f = {"auto": 0, "pair": ft.PAIR_TILES, "single": ft.SINGLE_TILES}[args.shape]
     f |= {"auto": 0, "deferred": ft.EPI_DEFERRED, "inline": ft.EPI_INLINE}[args.epilogue]
@@ -707,7 +712,7 @@ def run_single(args, ft, world, rank, local, secondary=False):
     refine_tc = bool(R) and args.refine_on == "tc"
     solver = ft.Solver([n], [mu], [kT], ms, mode=args.mode, want=3, flags=flags)
     if args.shape == "auto":
-        # tile shape: the library's autotuner times both shapes (untimed)
+        # tile shape: the library's autotuner times single CTAs and CTA pairs (untimed)
         shape, ms_single, ms_pair = solver.autotune(Hd, reps=2)
     else:
         shape, ms_single, ms_pair = solver.tile_shape()[0], None, None
@@ -824,7 +829,7 @@ def run_single(args, ft, world, rank, local, secondary=False):
         "data": "synthetic", "config": single_config(args),
         "details": {"mu": mu, "layers": L, "model": int(rec["model"]), "e_min": float(rec["e_min"]),
                     "e_max": float(rec["e_max"]), "beta_p": float(rec["beta_p"]),
-                    "tile_shape": {1: "256x256 CTA pairs", 0: "128x128 single CTAs", -1: "none"}[shape],
+                    "tile_shape": tile_label(solver, shape),
                     "epilogue": args.epilogue, "operands": args.operands, "launch": args.launch,
                     "autotune_ms": {"single": ms_single, "pair": ms_pair}},
         "tflops_alg": alg_flops / t_step / 1e12 * world,
@@ -1009,7 +1014,7 @@ def run_ragged(args, ft, world, rank, local, secondary=False):
         "details": {"instances_this_rank": len(ns), "valid_instances_this_rank": int(valid.sum()),
                     "sum_n3_this_rank": float(np.sum(n3)), "global_layers": lmax,
                     "models_used": {int(m): int(np.sum(rec["model"] == m)) for m in np.unique(rec["model"])},
-                    "tile_shape": {1: "256x256 CTA pairs", 0: "128x128 single CTAs", -1: "none"}[shape],
+                    "tile_shape": tile_label(solver, shape),
                     "autotune_ms": {"single": ms_single, "pair": ms_pair},
                     "timing": "CUDA-graph replays of one whole solve of the batch",
                     "eager_ms_per_step": t_eager * 1e3},

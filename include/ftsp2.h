@@ -79,12 +79,13 @@ typedef enum {
                                     FTSP2_E_VALIDITY and no result           */
 #define FTSP2_REFINE1       0x4  /* last layer in FTSP2_FP32 arithmetic       */
 #define FTSP2_REFINE2       0x8  /* last two layers in FTSP2_FP32 arithmetic  */
-/* Tile shape of the tensor-core layer launches.  By default a batch runs with
- * the shape ftsp2_autotune recorded for it or, if none was recorded, with the
- * shape a model of the layer's time prefers; these two flags override both. */
-#define FTSP2_PAIR_TILES    0x10 /* tiles on CTA pairs (cta_group::2): 256 rows by
-                                    256 or 128 columns, whichever the model of
-                                    the layer's time prefers                  */
+/* Tile shape of the tensor-core layer launches.  There are four: 128 x 128 and
+ * 128 x 64 tiles on single CTAs, 256 x 256 and 256 x 128 tiles on CTA pairs
+ * (cta_group::2).  By default a batch runs with the shape that a model of the
+ * layer's time prefers, among the two of the kind (single or pair) that
+ * ftsp2_autotune recorded for it or, if none was recorded, among all four; the
+ * flags override both. */
+#define FTSP2_PAIR_TILES    0x10 /* 256 x 256 tiles on CTA pairs               */
 #define FTSP2_SINGLE_TILES  0x20 /* 128 x 128 tiles on single CTAs             */
 /* Spectral bounds: by default the Gershgorin interval of Appendix A.  With this
  * flag it is tightened by 24 Lanczos steps in FP64 (start vector from
@@ -139,6 +140,9 @@ typedef enum {
  * end of every launch.  This flag forces one launch per layer (results are
  * identical). */
 #define FTSP2_LAYER_LAUNCHES 0x1000
+/* With FTSP2_PAIR_TILES or FTSP2_SINGLE_TILES: tiles of half as many columns
+ * (256 x 128, 128 x 64).  Without them no effect. */
+#define FTSP2_HALF_TILES     0x2000
 
 /* One Hamiltonian of a (ragged) batch.  H_b starts at dH + offset and is
  * n x n row-major; D_b starts at dD + offset.  Offsets are in elements. */
@@ -377,18 +381,19 @@ ftsp2_status ftsp2_density_mu(const double* dH, const ftsp2_instance* inst, ftsp
 
 /* ---- tile-shape autotuner ------------------------------------------------------ */
 
-/* Measures the batch with both tensor-core tile shapes and records the faster.
+/* Measures the batch with both kinds of tensor-core tiles, single CTAs and CTA
+ * pairs, each with the width that the time model prefers, and records the faster.
  * Arguments are those of ftsp2_density_entropy (the buffers are written as by
- * that call; the results of the last run are left in them).  For each shape
+ * that call; the results of the last run are left in them).  For each kind
  * the batch runs once untimed and then `reps` times between CUDA events on
- * `stream`; ms[0] receives the mean time of the 128 x 128 single-CTA shape,
- * ms[1] that of the pair shape (ms nullable), *choice the shape kept
+ * `stream`; ms[0] receives the mean time on single CTAs (128 x 128 or 128 x 64
+ * tiles), ms[1] that on pairs (256 x 256 or 256 x 128; ms nullable), *choice the kind kept
  * (0 single, 1 pair; -1 in FTSP2_FP32 mode, which has no tensor-core layers and
  * is not timed).  The record is keyed by device, mode, density/entropy
  * selection, refinement flags and the sorted list of orders n, lives for the
  * life of the process, and is shared by all threads (guarded by a mutex).
- * Synchronises `stream`.  Not usable during stream capture.  FTSP2_PAIR_TILES
- * and FTSP2_SINGLE_TILES in `flags` are ignored here.  Errors: those of
+ * Synchronises `stream`.  Not usable during stream capture.  FTSP2_PAIR_TILES,
+ * FTSP2_SINGLE_TILES and FTSP2_HALF_TILES in `flags` are ignored here.  Errors: those of
  * ftsp2_density_entropy; FTSP2_E_ARG if reps < 1. */
 ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst,
                             const ftsp2_instance* dInst, int nb,
@@ -397,13 +402,18 @@ ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst,
                             ftsp2_rescale_rec* dRec, void* ws, size_t ws_bytes,
                             int reps, int* choice, float* ms, void* stream);
 
-/* The tile shape a call with these arguments would use on the current device:
+/* The kind of tiles a call with these arguments would use on the current device:
  * 1 pair, 0 single, -1 none (FTSP2_FP32 mode).  `want` as in
  * ftsp2_workspace_size.  *from_tuner is set to 1 if the shape comes from an
  * ftsp2_autotune record, 0 if from the flags or the time model.  Host-only
  * apart from reading the device's SM count. */
 ftsp2_status ftsp2_tile_shape(const ftsp2_instance* inst, int nb, ftsp2_mode mode, int want,
                               int flags, int* shape, int* from_tuner);
+
+/* Rows and columns of those tiles (0 and 0 in FTSP2_FP32 mode).  Host-only, and
+ * without a look at the device when the flags force the shape. */
+ftsp2_status ftsp2_tile_size(const ftsp2_instance* inst, int nb, ftsp2_mode mode, int want,
+                             int flags, int* rows, int* cols);
 
 /* Forgets every ftsp2_autotune record. */
 ftsp2_status ftsp2_autotune_clear(void);

@@ -23,7 +23,7 @@ import ctypes as C
 import numpy as np
 
 from . import _lib
-from ._lib import (BF16X3, CLAMP, EPI_DEFERRED, EPI_INLINE, FP16X2, FP32, FULL_OPERANDS, LANCZOS, LAYER_LAUNCHES,
+from ._lib import (BF16X3, CLAMP, EPI_DEFERRED, EPI_INLINE, FP16X2, FP32, FULL_OPERANDS, HALF_TILES, LANCZOS, LAYER_LAUNCHES,
                    MIN_LAYERS, MODES,
                    PAIR_TILES,
                    REFINE1, REFINE2, REFINE_TC, SINGLE_TILES, SYNC,
@@ -36,7 +36,7 @@ __all__ = ["ModelSet", "Solver", "ftsp2_rescale", "ftsp2_train_coeffs", "ftsp2_t
            "ftsp2_train_normal_equations", "ftsp2_autotune_clear", "kernel_launch_count", "profile_layers",
            "set_wait_limit_ns", "wait_limit_ns", "debug_stall_layer",
            "profile_read", "MODES", "FP32", "TF32X3", "BF16X3", "FP16X2", "SYNC", "CLAMP", "REFINE1", "REFINE2",
-           "PAIR_TILES", "SINGLE_TILES", "LANCZOS", "MIN_LAYERS", "REFINE_TC", "EPI_DEFERRED", "EPI_INLINE", "FULL_OPERANDS", "LAYER_LAUNCHES", "TARGET_FERMI", "TARGET_ENTROPY", "Ftsp2Error", "status_string", "lib",
+           "PAIR_TILES", "SINGLE_TILES", "HALF_TILES", "LANCZOS", "MIN_LAYERS", "REFINE_TC", "EPI_DEFERRED", "EPI_INLINE", "FULL_OPERANDS", "LAYER_LAUNCHES", "TARGET_FERMI", "TARGET_ENTROPY", "Ftsp2Error", "status_string", "lib",
            "REC_DTYPE"]
 
 REC_DTYPE = np.dtype([("e_min", "f8"), ("e_max", "f8"), ("mu_p", "f8"), ("beta_p", "f8"), ("scale", "f8"),
@@ -334,10 +334,11 @@ class Solver:
         return D, T, S
 
     def autotune(self, H, reps=3, stream=None):
-        """ftsp2_autotune on this batch: times both tile shapes and records the
+        """ftsp2_autotune on this batch: times both kinds of tiles and records the
         faster for every later call with the same signature.  Returns
-        (shape, ms_single, ms_pair); shape 1 = 256 x 256 pairs, 0 = 128 x 128
-        single CTAs, -1 = no tensor-core layers (FP32 mode)."""
+        (shape, ms_single, ms_pair); shape 1 = CTA pairs (256 x 256 or 256 x 128
+        tiles, as the time model prefers), 0 = single CTAs (128 x 128 or
+        128 x 64), -1 = no tensor-core layers (FP32 mode)."""
         torch = _torch()
         if H.dtype != torch.float64 or not H.is_cuda or H.numel() < self.total:
             raise ValueError("H must be a CUDA float64 tensor with sum(n^2) elements")
@@ -356,6 +357,14 @@ class Solver:
         check(lib().ftsp2_tile_shape(self.host_inst, self.nb, self.mode, self.want, self.flags, C.byref(shape),
                                      C.byref(tuned)), "ftsp2_tile_shape")
         return shape.value, bool(tuned.value)
+
+    def tile_size(self):
+        """(rows, columns) of the tiles that run() uses (ftsp2_tile_size); (0, 0)
+        in FP32 mode."""
+        rows, cols = C.c_int(), C.c_int()
+        check(lib().ftsp2_tile_size(self.host_inst, self.nb, self.mode, self.want, self.flags, C.byref(rows),
+                                    C.byref(cols)), "ftsp2_tile_size")
+        return rows.value, cols.value
 
     def records(self):
         raw = self.rec.cpu().numpy()

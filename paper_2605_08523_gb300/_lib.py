@@ -20,7 +20,7 @@ MODES = {"fp32": FP32, "tf32x3": TF32X3, "bf16x3": BF16X3, "fp16x2": FP16X2}
 SYNC, CLAMP, REFINE1, REFINE2, PAIR_TILES, SINGLE_TILES, LANCZOS, MIN_LAYERS, REFINE_TC = \
     0x1, 0x2, 0x4, 0x8, 0x10, 0x20, 0x40, 0x80, 0x100
 EPI_DEFERRED, EPI_INLINE, FULL_OPERANDS = 0x200, 0x400, 0x800
-LAYER_LAUNCHES = 0x1000
+LAYER_LAUNCHES, HALF_TILES = 0x1000, 0x2000
 FAMILY_MLSP2, FAMILY_SKIP, FAMILY_MAX = 0, 1, 2
 TARGET_FERMI, TARGET_ENTROPY = 0, 1
 
@@ -74,6 +74,7 @@ SIGNATURES = {
     "ftsp2_autotune": (_I, [_VP, _PINST, _VP, _I, _VP, _I, _I, _VP, _VP, _VP, _VP, _VP, _SZ, _I,
                             C.POINTER(_I), C.POINTER(C.c_float), _VP]),
     "ftsp2_tile_shape": (_I, [_PINST, _I, _I, _I, _I, C.POINTER(_I), C.POINTER(_I)]),
+    "ftsp2_tile_size": (_I, [_PINST, _I, _I, _I, _I, C.POINTER(_I), C.POINTER(_I)]),
     "ftsp2_autotune_clear": (_I, []),
     "ftsp2_train_workspace_size": (_SZ, [_I, _I]),
     "ftsp2_train_coeffs": (_I, [_I, _D, _D, _I, _D, _I, C.c_uint64, _I, _I, C.POINTER(_D), C.POINTER(_D),

@@ -530,11 +530,11 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
 static ftsp2_status from_cuda(cudaError_t e) { return e == cudaSuccess ? FTSP2_OK : FTSP2_E_CUDA; }
 
 // ---- tile-shape choice --------------------------------------------------------
-// Tensor-core layers run on single CTAs with 128 x 128 tiles or on CTA pairs with
-// 256 x 256 or 256 x 128 tiles.  Single or pair is forced by a flag, or recorded
-// by ftsp2_autotune per batch signature (device, mode, chains, refinement, the
-// sorted list of orders n); otherwise, and for the width of the pair tiles, the
-// cost model below decides.
+// Tensor-core layers run on single CTAs with 128 x 128 or 128 x 64 tiles or on CTA pairs with
+// 256 x 256 or 256 x 128 tiles.  A shape is forced by flags; single or pair is
+// recorded by ftsp2_autotune per batch signature (device, mode, chains, refinement,
+// the sorted list of orders n); otherwise, and for the width of a recorded kind's
+// tiles, the cost model below decides.
 static std::mutex g_tune_mu;
 static std::map<uint64_t, int> g_tune;
 
@@ -615,6 +615,19 @@ static double shape_cost(const ftsp2_instance* inst, int nb, int nch, int mode, 
     return load / units + (nb * nch == 1 ? 0.5 : 0.35) * load / tiles;
 }
 
+// The shape that the flags force (-1: none) and the flags that force a shape.
+static int forced_shape(int flags) {
+    const bool half = (flags & FTSP2_HALF_TILES) != 0;
+    if (flags & FTSP2_PAIR_TILES) return half ? SHAPE_PAIR128 : SHAPE_PAIR;
+    if (flags & FTSP2_SINGLE_TILES) return half ? SHAPE_SINGLE64 : SHAPE_SINGLE;
+    return -1;
+}
+constexpr int kShapeFlags = FTSP2_PAIR_TILES | FTSP2_SINGLE_TILES | FTSP2_HALF_TILES;
+static int flags_of_shape(int shape) {
+    return (tc_pair(shape) ? FTSP2_PAIR_TILES : FTSP2_SINGLE_TILES) |
+           (shape == SHAPE_PAIR128 || shape == SHAPE_SINGLE64 ? FTSP2_HALF_TILES : 0);
+}
+
 // The forced or recorded choice of a call: 1 pair, 0 single, -1 neither.
 static int chosen_pair(const ftsp2_instance* inst, int nb, int mode, int want, int flags, int* from_tuner = nullptr) {
     if (from_tuner) *from_tuner = 0;
@@ -627,12 +640,12 @@ static int chosen_pair(const ftsp2_instance* inst, int nb, int mode, int want, i
     return it->second;
 }
 
-// Shape of a call's tensor-core layers: the cheapest by the model within the
-// forced or recorded choice (pair < 0: none).  Pair tiles forced together with a
-// placement of their final epilogue are the 256 x 256 ones, which have the choice.
+// Shape of a call's tensor-core layers: the forced one, or the cheapest by the
+// model within the recorded choice (pair < 0: none).
 static int layer_shape(const ftsp2_instance* inst, int nb, int mode, int want, int flags, int pair, int sms,
                        bool deferred) {
-    if ((flags & FTSP2_PAIR_TILES) && (flags & (FTSP2_EPI_DEFERRED | FTSP2_EPI_INLINE))) return SHAPE_PAIR;
+    const int forced = forced_shape(flags);
+    if (forced >= 0) return forced;
     const int nch = want == 3 ? 2 : 1;
     int best = -1;
     double cost = 0.0;
@@ -1361,6 +1374,14 @@ ftsp2_status ftsp2_density_mu(const double* dH, const ftsp2_instance* inst, ftsp
     }
 }
 
+static ftsp2_status sm_count(int& sms) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return FTSP2_E_CUDA;
+    return FTSP2_OK;
+}
+
 static int want_of(const float* dD, const double* dTrace, const double* dS) {
     if (!dS) return 1;
     if (!dD && !dTrace) return 2;
@@ -1374,7 +1395,7 @@ ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst, const 
     if (reps < 1 || !choice) return FTSP2_E_ARG;
     if (nb < 1 || !inst) return FTSP2_E_ARG;
     if (ms) ms[0] = ms[1] = 0.f;
-    const int base = flags & ~(FTSP2_PAIR_TILES | FTSP2_SINGLE_TILES | FTSP2_SYNC);
+    const int base = flags & ~(kShapeFlags | FTSP2_SYNC);
     if (mode == FTSP2_FP32) {
         *choice = -1;
         return ftsp2_density_entropy(dH, inst, dInst, nb, set, mode, base | FTSP2_SYNC, dD, dTrace, dS, dRec, ws,
@@ -1387,9 +1408,12 @@ ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst, const 
         return FTSP2_E_CUDA;
     }
     float t[2] = {0.f, 0.f};
-    ftsp2_status st = FTSP2_OK;
-    for (int shape = 0; shape < 2 && st == FTSP2_OK; ++shape) {
-        const int f = base | (shape ? FTSP2_PAIR_TILES : FTSP2_SINGLE_TILES);
+    int sms = 0;
+    ftsp2_status st = sm_count(sms);
+    for (int pair = 0; pair < 2 && st == FTSP2_OK; ++pair) {
+        // the shape that a record of this kind leads to
+        const int f = base | flags_of_shape(layer_shape(inst, nb, mode, want_of(dD, dTrace, dS), base, pair, sms,
+                                                        deferred_epilogue(inst, nb, base)));
         // untimed run with FTSP2_SYNC: surfaces per-instance errors once
         st = ftsp2_density_entropy(dH, inst, dInst, nb, set, mode, f | FTSP2_SYNC, dD, dTrace, dS, dRec, ws,
                                    ws_bytes, stream);
@@ -1400,11 +1424,11 @@ ftsp2_status ftsp2_autotune(const double* dH, const ftsp2_instance* inst, const 
                                        stream);
         if (st != FTSP2_OK) break;
         if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&t[shape], e0, e1) != cudaSuccess) {
+            cudaEventElapsedTime(&t[pair], e0, e1) != cudaSuccess) {
             st = FTSP2_E_CUDA;
             break;
         }
-        t[shape] /= (float)reps;
+        t[pair] /= (float)reps;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1430,13 +1454,33 @@ ftsp2_status ftsp2_tile_shape(const ftsp2_instance* inst, int nb, ftsp2_mode mod
         *shape = -1;
         return FTSP2_OK;
     }
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return FTSP2_E_CUDA;
+    int sms = 0;
+    const ftsp2_status st = sm_count(sms);
+    if (st != FTSP2_OK) return st;
     const int pair = chosen_pair(inst, nb, mode, want, flags, from_tuner);
     *shape = layer_shape(inst, nb, mode, want, flags, pair, sms, deferred_epilogue(inst, nb, flags));
     *shape = tc_pair(*shape) ? 1 : 0;
+    return FTSP2_OK;
+}
+
+ftsp2_status ftsp2_tile_size(const ftsp2_instance* inst, int nb, ftsp2_mode mode, int want, int flags, int* rows,
+                             int* cols) {
+    if (!inst || nb < 1 || !rows || !cols || want < 1 || want > 3 || mode < FTSP2_FP32 || mode > FTSP2_FP16X2)
+        return FTSP2_E_ARG;
+    if (mode == FTSP2_FP32) {
+        *rows = *cols = 0;
+        return FTSP2_OK;
+    }
+    int shape = forced_shape(flags);
+    if (shape < 0) {
+        int sms = 0;
+        const ftsp2_status st = sm_count(sms);
+        if (st != FTSP2_OK) return st;
+        shape = layer_shape(inst, nb, mode, want, flags, chosen_pair(inst, nb, mode, want, flags), sms,
+                            deferred_epilogue(inst, nb, flags));
+    }
+    *rows = tc_block_m(shape);
+    *cols = tc_block_n(shape);
     return FTSP2_OK;
 }
 

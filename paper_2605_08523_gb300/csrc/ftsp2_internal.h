@@ -290,8 +290,8 @@ struct LayerMaps {
 };
 
 // Tensor-core layer (k_layer_tc.cu); mode in {TF32X3, BF16X3, FP16X2}; shape 0:
-// 128 x 128 tiles on single CTAs (units = CTAs), 1: 256 x 256 and 2: 256 x 128
-// tiles on CTA pairs (units = pairs).  Persistent grid of `units`.
+// 128 x 128 and 3: 128 x 64 tiles on single CTAs (units = CTAs), 1: 256 x 256 and
+// 2: 256 x 128 tiles on CTA pairs (units = pairs).  Persistent grid of `units`.
 enum { SHAPE_SINGLE = 0, SHAPE_PAIR = 1, SHAPE_PAIR128 = 2, SHAPE_SINGLE64 = 3 };
 constexpr int kShapes = 4;
 constexpr bool tc_pair(int shape) { return shape == SHAPE_PAIR || shape == SHAPE_PAIR128; }
