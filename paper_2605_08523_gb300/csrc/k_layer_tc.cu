@@ -55,11 +55,15 @@
 //                operands).  It is a chain of short dependent steps (a warp issues
 //                an instruction every eleven clocks), so FP16X2 operands of
 //                128-column tiles have 16 warps of 32 columns (96 registers) and
-//                the others 8 warps of 64 or 128 columns (168 registers): the
-//                wider formats' planes do not fit in 96.  8 -> 16 warps, FP16X2:
-//                n = 256 277 -> 261 us, 60 fragments 411 -> 380, ragged batch
-//                22.8 -> 22.1 ms, n = 1501 unchanged; BF16X3 and TF32X3 0.7 %
-//                slower at n = 1024 and 2048.
+//                256-column tiles 16 warps of 64; the others have 8 warps of 64
+//                columns (168 registers), 128 at the last layer: there the wider
+//                formats' planes spill in 96.  8 -> 16 warps, FP16X2: n = 256
+//                277 -> 261 us, 60 fragments 411 -> 380, ragged batch 22.8 ->
+//                22.1 ms, n = 1501 unchanged; BF16X3 and TF32X3 on 128 columns
+//                0.7 % slower at n = 1024 and 2048.  256 x 256 tiles, inline, 8 ->
+//                16 warps with the state 16 columns ahead: n = 2200 TF32X3
+//                (density) 2173 -> 2038 us, n = 2700 FP16X2 1526 -> 1456, n = 2816
+//                FP16X2 (density + entropy) 2716 -> 2546.
 //   last warp  : context warp (below)
 // The loops of warps 0 and 1 run on the whole warp with one elected lane issuing:
 // their values are then uniform, and a copy or an MMA takes no moves from vector
@@ -79,7 +83,11 @@
 // and go on with the next tile at once; two store warps stream scratch, Z_k and
 // A_k through a small shared ring (cp.async) and run the final epilogue while the
 // next tile's MMAs run.  A unit's last tile runs inline, so no store-warp tail
-// follows the last MMAs.
+// follows the last MMAs.  At 96 registers a thread (640 threads) the epilogue has
+// 16 columns of the state at a time and its context in shared memory; with 32
+// columns and a context in registers it spilled 640 bytes for 390 (FP16X2), and
+// n = 2816 (density + entropy, deferred) took 2810 us, 2431 now, n = 5000 TF32X3
+// (density) 11585, 11340 now.
 //
 // Multi-layer launches (a.nlayers > 1).  The work items are (layer, tile) in
 // layer order; every role walks the same item sequence.  An item of layer g
@@ -150,7 +158,7 @@ constexpr int kCtaRows = 128;
 template <int OUTFMT, int SHAPE>
 constexpr int epi_warps() {
     if (SHAPE == SHAPE_SINGLE64) return OUTFMT == -1 ? 4 : 8;     // last layer: a 32 x 64 block of partial sums a warp
-    return OUTFMT == OP_F16X2 && SHAPE != SHAPE_PAIR ? 16 : 8;
+    return OUTFMT != -1 && (OUTFMT == OP_F16X2 || SHAPE == SHAPE_PAIR) ? 16 : 8;
 }
 template <int OUTFMT, int SHAPE>
 constexpr int tc_threads() { return 32 * (2 + epi_warps<OUTFMT, SHAPE>() + 1); }
@@ -758,11 +766,14 @@ struct State {
 };
 using State32 = State<2>;
 
-// One 32 x 32 block: v holds the sums S of the lane's row.
-template <int FMT, bool CAN_RESIDE, int H>
+// One 32 x 32 block: v holds the sums S of the lane's row, s the state of its 32
+// columns (H = 2) or of the first 16 (H = 1).  fetch(h) follows the use of half h:
+// it loads that half of the next block (H = 2), or the second half of this block
+// (h = 0) and the first one of the next (h = 1).
+template <int FMT, bool CAN_RESIDE, int H, class Fetch>
 __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c, const CUtensorMap* wmaps, Stager& st,
                                             int R0, int c0, uint32_t tstate, bool from_tmem, bool to_tmem,
-                                            float (&v)[32], State<H>& s, int c_next) {
+                                            float (&v)[32], State<H>& s, Fetch&& fetch) {
     constexpr int NPL = OpFmtT<FMT>::NPL;
     const int n = c.n, r = R0 + st.lane;
     const float mul = c.mul, bp = c.bp, d = c.d;
@@ -805,12 +816,7 @@ __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c
                 }
             }
         }
-        if constexpr (H == 2) {
-            // the same columns of the next block
-            if (!from_tmem && c_next >= 0) load16(a, c.Z, n, R0, r, c_next + 16 * h, s.z[h], s.x[h]);
-        } else if (h == 0 && !from_tmem) {
-            load16(a, c.Z, n, R0, r, c0 + 16, s.z[0], s.x[0]);
-        }
+        fetch(h);
     }
     if (!(R0 + 31 < n && c0 + 31 < n)) {
         // zeros in the padding
@@ -1424,7 +1430,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
                 for (int h = 0; h < AH; ++h) load16(a, c.Z, n, R0, R0 + lane, C0 + cb0 + 16 * h, s.z[h], s.x[h]);
             };
             // Chunk drain: every chunk is added into acc and its buffer released.
-            // The 128 columns of a 256-column tile's warp leave no registers for
+            // The columns of a 256-column tile's warp leave no registers for
             // the final epilogue: there the finished sum is written back into the
             // last chunk's buffer, which stays held, and read from it block by
             // block; the MMAs of the next tile meanwhile fill the other buffer.
@@ -1473,7 +1479,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
             // every block of the warp: its sums in v, the state loaded ahead in s
             auto blocks = [&](auto&& block) {
                 if constexpr (HOLD) {
-                    State32 s;
+                    State<AH> s;
                     load_first(s);
                     const uint32_t tfin = tlane + (uint32_t)(buf * TN);
 #pragma unroll 1
@@ -1499,8 +1505,18 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
                 if (live && work) {
                     const CUtensorMap* const wm = (c.maps ? wmaps1 : wmaps0).w[c.chain];
                     blocks([&](int cb, float (&v)[32], State<AH>& s) {
-                        epi_block32<OUTFMT, CAN_RESIDE, AH>(a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem,
-                                                        to_tmem, v, s, next_of(cb));
+                        epi_block32<OUTFMT, CAN_RESIDE, AH>(
+                            a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem, to_tmem, v, s, [&](int h) {
+                                const int cn = EPI_COLS > 32 ? next_of(cb) : -1;
+                                if (from_tmem) return;
+                                if constexpr (AH == 2) {
+                                    if (cn >= 0) load16(a, c.Z, n, R0, R0 + lane, cn + 16 * h, s.z[h], s.x[h]);
+                                } else if (h == 0) {
+                                    load16(a, c.Z, n, R0, R0 + lane, C0 + cb + 16, s.z[0], s.x[0]);
+                                } else if (cn >= 0) {
+                                    load16(a, c.Z, n, R0, R0 + lane, cn, s.z[0], s.x[0]);
+                                }
+                            });
                     });
                     if (CAN_RESIDE && to_tmem) tmem_wait_st();
                 }
@@ -1898,22 +1914,25 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                     int en = e;
                     const bool next = next_block(c, sw, en);
                     float v[32];
-                    State32 s;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
+                    State<1> s;
+                    // half h of the block from the ring, whose entry takes that of the next one
+                    auto take = [&](int h) {
                         // oldest copy group first: the other half, or the next block's first half
                         if (h == 0 || next) cp_async_wait<1>();
                         else cp_async_wait<0>();
                         const float* const src = reinterpret_cast<const float*>(ring + h * kEntryBytes) + lane * 4;
                         load_state8(src, v + 16 * h);
                         load_state8(src + 256, v + 16 * h + 8);
-                        load_state8(src + 512, s.z[h]);
-                        load_state8(src + 768, s.z[h] + 8);
-                        load_state8(src + 1024, s.x[h]);
-                        load_state8(src + 1280, s.x[h] + 8);
+                        load_state8(src + 512, s.z[0]);
+                        load_state8(src + 768, s.z[0] + 8);
+                        load_state8(src + 1024, s.x[0]);
+                        load_state8(src + 1280, s.x[0] + 8);
                         if (next) issue(en, h, h);
-                    }
-                    epi_block32<OUTFMT, false>(a, c, wm, st, d.R0, d.c0, 0u, false, false, v, s, -1);
+                    };
+                    take(0);
+                    epi_block32<OUTFMT, false>(a, c, wm, st, d.R0, d.c0, 0u, false, false, v, s, [&](int h) {
+                        if (h == 0) take(1);
+                    });
                     e = en;
                     more = next;
                 }
@@ -1944,9 +1963,8 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
             item_of(a, f, g, t);
             // Only the chunk count and the liveness of the warp's block are
             // carried through the drain loop; the tile's descriptor and the
-            // rest of the context are fetched again for the final epilogue
-            // (keeps the drain loop of a pair tile, with its 64 accumulator
-            // registers, free of spills).
+            // rest of the context are fetched again for the final epilogue, into
+            // shared memory (the 64 accumulators leave 32 registers).
             int nch;
             bool warp_live, defer_tile;
             {
@@ -2035,10 +2053,16 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
             }
             if (warp_live && work) {
                 // The unit's last tile: its MMAs have all completed and no loads
-                // follow, so the blocks are staged in the operand ring.
-                ItemCtx c;
-                const InstWork& w = a.iw[tl.inst];
-                fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], (int)rank, c);
+                // follow, so the blocks are staged in the operand ring, with the
+                // warp's context behind them.
+                ItemCtx& c = *reinterpret_cast<ItemCtx*>(smem + kDeferWarps * kStageBytes + (warp - 2) * 256);
+                static_assert(sizeof(ItemCtx) <= 256 && kDeferWarps * (kStageBytes + 256) <= C::STAGES * STAGE_BYTES,
+                              "staging and contexts in the ring");
+                if (lane == 0) {
+                    const InstWork& w = a.iw[tl.inst];
+                    fill_epilogue<MODE, OUTFMT, SHAPE_PAIR>(a, tl, w, a.layers[w.layer_off[tl.chain] + k], (int)rank, c);
+                }
+                __syncwarp();
                 Stager st{smem_u32(smem) + (uint32_t)((warp - 2) * kStageBytes), lane, 0, 2};
                 const CUtensorMap* const wm = (((g - a.gl) & 1) ? wmaps1 : wmaps0).w[tl.chain];
                 const int R0 = c.row0 + q * 32;
@@ -2047,12 +2071,13 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                     const int c0 = c.col0 + cq * EPI_COLS + cb;
                     if (!(c0 >= R0 && c0 < c.n)) continue;
                     float v[32];
-                    State32 s;
+                    State<1> s;
                     load16(a, c.Z, c.n, R0, R0 + lane, c0, s.z[0], s.x[0]);
-                    load16(a, c.Z, c.n, R0, R0 + lane, c0 + 16, s.z[1], s.x[1]);
                     tmem_ld32(tfin + cb, reinterpret_cast<uint32_t*>(v));
                     tmem_wait_ld();
-                    epi_block32<OUTFMT, false>(a, c, wm, st, R0, c0, 0u, false, false, v, s, -1);
+                    epi_block32<OUTFMT, false>(a, c, wm, st, R0, c0, 0u, false, false, v, s, [&](int h) {
+                        if (h == 0) load16(a, c.Z, c.n, R0, R0 + lane, c0 + 16, s.z[0], s.x[0]);
+                    });
                 }
                 st.finish();
             }
