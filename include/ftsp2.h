@@ -119,7 +119,8 @@ typedef enum {
  * most 192 CTAs) and go on with the next tile, so that the epilogue's memory
  * traffic overlaps the next tile's MMAs; for shorter tiles the accumulating
  * warps run it inline.  These two flags force one or the other (results are
- * identical). */
+ * identical), and have a call that runs on pairs do so with 256 x 256 tiles: unless
+ * FTSP2_HALF_TILES is given, and without effect on single CTAs. */
 #define FTSP2_EPI_DEFERRED  0x200
 #define FTSP2_EPI_INLINE    0x400
 /* Operand storage of the FP16X2 / BF16X3 tensor-core layers.  The square of a

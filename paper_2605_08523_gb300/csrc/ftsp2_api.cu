@@ -646,6 +646,12 @@ static int layer_shape(const ftsp2_instance* inst, int nb, int mode, int want, i
                        bool deferred) {
     const int forced = forced_shape(flags);
     if (forced >= 0) return forced;
+    // Only 256 x 256 tiles have a choice of where their final epilogue runs: a call
+    // that asks for one gets them wherever the padding model, or its record, has pairs
+    if (flags & (FTSP2_EPI_DEFERRED | FTSP2_EPI_INLINE)) {
+        if (pair < 0) pair = chunk_shape(inst, nb, sms);
+        if (pair) return SHAPE_PAIR;
+    }
     const int nch = want == 3 ? 2 : 1;
     int best = -1;
     double cost = 0.0;
