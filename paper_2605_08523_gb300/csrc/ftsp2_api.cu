@@ -582,37 +582,57 @@ static int chunk_shape(const ftsp2_instance* inst, int nb, int sms) {
     return cost[1] <= cost[0] ? 1 : 0;
 }
 
-// Clocks of one layer with a tile shape, from the measured parts of a tile: the
-// K loop per 64 elements (the MMAs of a pair: 768 clocks of FP16X2 on 128
-// columns run in 850, on 256 columns 1536 in 1570; a single CTA's 128 x 128
-// MMAs, both panels from one shared memory, take 1300 for 768, its 128 x 64 ones
-// 1000 for 384), and the final epilogue, which follows the K loop when a unit has
-// one tile and otherwise overlaps the next tile's (kStream is then its share of a
-// tile, bound by the chain of its steps).  With more tiles than units the layer
-// costs its mean load, and a part of a tile for the uneven end: less when other
-// instances or chains fill it.  Measured (us per solve; 128 x 128 / 256 x 128 /
-// 128 x 64), one lattice, density + entropy, FP16X2: n = 64: 149 / 154 / 136; 384:
-// 268 / 266 / 230; 900: 442 / 394 / 393; 1280: 545 / 479 / 569; 1800: 1095 / 982 /
-// 1345; density, TF32X3: n = 128: 307 / 299 / 213; 900: 730 / 608 / 560; 1536:
-// 1026 / 823 / 1491; 24 fragments of 16 to 200: 497 / 491 / 470; 40 instances of
-// n = 256: 603 / 706 / 632; the ragged batch of 512: 21520 / 24830 / 23080.  256 x
-// 256 pays from n = 3000 to 4000 on (4096: 9175 / 7731, 256 x 256 7388).
+// Clocks of one layer with a tile shape.  Where every unit has at most one tile it is
+// the latency of a tile: its K loop, kAlone clocks per 64 elements of K, and its
+// final epilogue (kEpilogue).  With more tiles the loops run at kBusy clocks, under
+// the power limit and beside other tiles' epilogues, and a tile takes at least
+// kStream, the chain of its epilogue's steps, which the next tile's loop hides; the
+// 256 x 256 tiles' inline epilogue holds one of two accumulators and adds to the
+// loop instead.  One matrix and one chain run in whole waves, since a layer waits
+// for all tiles of the one before (128 x 64 tiles then never pay); several fill each
+// other's waves, but for an uneven end that shrinks with their number, and take at
+// least a tile's latency, kBeside more with the state in memory.
+// The constants are fitted to the times of the four shapes, forced, in 470 cases of
+// one matrix (n = 130 to 5500) and 229 of a ragged batch (2 to 512 instances), all
+// modes, one and two chains: on average the shape taken is 0.2 % slower than the
+// best one, and 9 % at most; with the constants of a tile alone in both regimes it
+// was 2.3 % and 30 %.  us per solve (128 x 128 / 256 x 256 / 256 x 128 / 128 x 64):
+//   n =  520 FP16X2 D      323 /     - /   305 /  276   128 x 64
+//   n = 1537 FP16X2 D      622 /  1021 /   529 /  900   256 x 128
+//   n = 2560 FP16X2 D     1753 /  1349 /  1454 /    -   256 x 256: one wave for two
+//   n = 2976 BF16X3 D     3159 /  4610 /  3633 /    -   128 x 128: two waves for three
+//   n = 3456 TF32X3 D + S    - /  7354 /  8701 /    -   256 x 256
+//   n = 4400 BF16X3 D + S    - / 15112 / 17717 /    -   256 x 256
+//   n = 5000 TF32X3 D        - / 11881 / 12807 /    -   256 x 256
+//   100 instances of 128, FP16X2 D           461 /  714 /  539 /  476   128 x 128
+//   100 instances of 128, TF32X3 D           493 /  792 /  619 /  409   128 x 64
+//   80 instances of 32 to 469, FP16X2 D + S  1745 / 2440 / 2150 / 1997   128 x 128
 static double shape_cost(const ftsp2_instance* inst, int nb, int nch, int mode, int sms, int shape, bool deferred) {
-    static const double kSlice[3][kShapes] = {{2860, 3140, 1700, 1750}, {2500, 3100, 1650, 1700}, {1300, 1570, 850, 1000}};   // TF32X3, BF16X3, FP16X2
-    const double slice = kSlice[mode == FTSP2_TF32X3 ? 0 : mode == FTSP2_BF16X3 ? 1 : 2][shape];
-    const double epi = shape == SHAPE_SINGLE ? 7000 : shape == SHAPE_PAIR128 ? 7700 : shape == SHAPE_SINGLE64 ? 5000 : 28000;
-    const double stream = shape == SHAPE_PAIR && !deferred ? 28000 : shape == SHAPE_SINGLE64 ? 9000 : 14000;
+    // [TF32X3, BF16X3, FP16X2][128 x 128, 256 x 256, 256 x 128, 128 x 64]
+    static const double kAlone[3][kShapes] = {{2620, 2760, 1430, 1420}, {2720, 4990, 1690, 1560}, {1160, 1300, 725, 1020}};
+    static const double kBusy[3][kShapes] = {{2240, 2520, 1590, 1160}, {1890, 2270, 1460, 1510}, {1210, 1270, 895, 858}};
+    // the 128-column tiles have sixteen epilogue warps for FP16X2, else eight
+    static const double kStream[3][kShapes] = {{13100, 14000, 22200, 5960}, {13100, 14000, 22200, 5960}, {8660, 14000, 20000, 5960}};
+    static const double kEpilogue[kShapes] = {7360, 31500, 9670, 4940}, kBeside[kShapes] = {2860, 2600, 2470, 2920};
+    static const double kEnd[kShapes] = {0.55, 0.37, 0.39, 0.56};
+    constexpr double kInline = 15000, kInlineMin = 20200, kChainEnd = 3.07;
+    const int m = mode == FTSP2_TF32X3 ? 0 : mode == FTSP2_BF16X3 ? 1 : 2;
     const double units = std::max(1, tc_pair(shape) ? sms / 2 : sms);
-    double tiles = 0.0, load = 0.0, longest = 0.0;
+    double tiles = 0.0, load = 0.0, alone = 0.0, longest = 0.0;
     for (int b = 0; b < nb; ++b) {
         const double t = (double)nch * (double)host_tiles_of(inst[b].n, tc_block_m(shape), tc_block_n(shape));
-        const double k = slice * std::ceil(inst[b].n / 64.0);
+        const double nk = std::ceil(inst[b].n / 64.0), k = kBusy[m][shape] * nk;
+        const double tile =
+            shape == SHAPE_PAIR && !deferred ? std::max(k + kInline, kInlineMin) : std::max(k, kStream[m][shape]);
         tiles += t;
-        load += t * std::max(k, stream);
-        longest = std::max(longest, k);
+        load += t * tile;
+        alone = std::max(alone, kAlone[m][shape] * nk + kEpilogue[shape]);
+        longest = std::max(longest, tile);
     }
-    if (tiles <= units) return longest + epi;
-    return load / units + (nb * nch == 1 ? 0.5 : 0.35) * load / tiles;
+    if (tiles <= units) return alone;
+    if (nb * nch == 1)
+        return shape == SHAPE_SINGLE64 ? HUGE_VAL : std::ceil(tiles / units) * longest + kChainEnd * kEpilogue[shape];
+    return std::max(load / units, alone + kBeside[shape]) + kEnd[shape] * load / tiles / std::sqrt((double)nb * nch);
 }
 
 // The shape that the flags force (-1: none) and the flags that force a shape.

@@ -70,13 +70,13 @@ def test_four_shapes_bitwise(ft, mode, extra, ns):
                                      ([65 + (37 * i) % 64 for i in range(70)], 3)],
                          ids=["100x128", "140x96", "60x100", "70x65-128"])
 def test_one_square_tile_per_cta(ft, mode, ns, want):
-    """Batches with one 128 x 128 tile per CTA, which run on those by default: B read
-    from A's panel, the state in TMEM and the operands staged in the ring."""
+    """Batches with one 128 x 128 tile per CTA, which run on those by default in FP16X2
+    mode: B read from A's panel, the state in TMEM and the operands staged in the ring."""
     Hs = matrices(ns, 23)
     Hd = torch.from_numpy(wl.pack_batch(Hs)[0]).cuda()
-    s = solve(ft, ns, mode, 0, Hd, want)
+    s = solve(ft, ns, mode, 0 if mode == "fp16x2" else ft.SINGLE_TILES, Hd, want)
     assert s.tile_size() == (128, 128)
-    for flags in (ft.PAIR_TILES, ft.LAYER_LAUNCHES, ft.SINGLE_TILES | ft.HALF_TILES):
+    for flags in (ft.PAIR_TILES, 0, ft.SINGLE_TILES | ft.LAYER_LAUNCHES, ft.SINGLE_TILES | ft.HALF_TILES):
         assert same(s, solve(ft, ns, mode, flags, Hd, want)), flags
     for b in (0, len(ns) // 2, len(ns) - 1):
         ex = pipeline.method_exact(Hs[b], 0.1, 0.15, [PRINTED])
