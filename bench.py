@@ -673,16 +673,17 @@ def cpu_baseline(args, reps=3):
 # ---------------------------------------------------------------------------
 # our arm: one matrix per rank
 # ---------------------------------------------------------------------------
-def hw_flops_per_solve(n, T, L, R, mode, refine_tc, chains=2):
-    """(tensor MMA flops a solve issues, tensor-core layers): upper-triangle
-    tiles of side T, each T x T x n per product; 3 products per FP16X2 / TF32X3
+def hw_flops_per_solve(n, tile, L, R, mode, refine_tc, chains=2):
+    """(tensor MMA flops a solve issues, tensor-core layers): the tiles (rows,
+    columns) that touch the upper triangle, rows x columns x n per product; 3 products per FP16X2 / TF32X3
     layer, 6 per BF16X3 layer; refinement layers on the tensor cores are BF16X3
     (in BF16X3 mode they are ordinary layers), on the CUDA cores they issue no
     MMAs."""
     if mode == "fp32":
         return 0.0, 0
-    nt = math.ceil(n / T)
-    per_product = 2.0 * (nt * (nt + 1) // 2) * T * T * n * chains
+    rows, cols = tile
+    tiles = sum(min(math.ceil((J + 1) * cols / rows), math.ceil(n / rows)) for J in range(math.ceil(n / cols)))
+    per_product = 2.0 * tiles * rows * cols * n * chains
     nprod = {"fp16x2": 3, "tf32x3": 3, "bf16x3": 6}[mode]
     if refine_tc and mode == "bf16x3":
         R = 0
@@ -805,7 +806,7 @@ def run_single(args, ft, world, rank, local, secondary=False):
     pk, pk_kind = peaks()
     # mean time of one tensor-core layer: the profiled launches cover every
     # tensor-core layer of the steps (a multi-layer launch counts its layers)
-    hw_solve, tc_layers = hw_flops_per_solve(n, 256 if shape == 1 else 128, L, R, args.mode, refine_tc)
+    hw_solve, tc_layers = hw_flops_per_solve(n, solver.tile_size(), L, R, args.mode, refine_tc)
     layer_avg = layer_ms / max(1, args.steps * tc_layers) / 1000.0
     alg_per_launch = 2 * float(n) ** 3          # one layer of both chains: n^3 per chain
     achieved = alg_per_launch / layer_avg / 1e12 if layer_avg > 0 else None
