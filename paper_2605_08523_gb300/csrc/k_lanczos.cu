@@ -33,6 +33,7 @@
 // checked against the eigenvalues of the workload families in the tests.
 #include <algorithm>
 
+#include "div_by.h"
 #include "ftsp2_internal.h"
 
 namespace ftsp2 {
@@ -62,14 +63,6 @@ __device__ double block_sum(double v, double* sh) {
     s = sh[T / 32];
     __syncthreads();
     return s;
-}
-
-// w / b with r = 1 / b: one correction of the product (Markstein's division step)
-// instead of a full division, some 20 instructions of the FP64 pipe (16 clocks a
-// warp instruction) each.
-__device__ __forceinline__ double div_by(double w, double b, double r) {
-    const double q = w * r;
-    return fma(fma(-q, b, w), r, q);
 }
 
 __device__ __forceinline__ double* lz_vec(const LanczosArgs& a, int which, int b) {
