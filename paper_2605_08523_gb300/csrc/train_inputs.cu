@@ -25,7 +25,6 @@
 #include <cmath>
 #include <cstdint>
 #include <memory>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -50,7 +49,7 @@ static void parallel_ranges(int n, const F& body) {
     int here = 1;                             // part 0 and those from `here` on run in this thread
     try {
         for (; here < parts; ++here) th[here] = std::thread(part, here);
-    } catch (const std::system_error&) {
+    } catch (...) {                           // no thread, or no memory for one
     }
     part(0);
     for (int i = here; i < parts; ++i) part(i);
