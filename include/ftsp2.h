@@ -633,7 +633,7 @@ uint64_t ftsp2_kernel_launch_count(void);
  * has finished) and of the kernel's internal pipeline barriers.  When a
  * dependency wait runs out, the kernel records FTSP2_E_TIMEOUT in the call's
  * status word and every CTA finishes its work list in a skip mode that keeps
- * the barrier protocol (no loads, MMAs or stores), so nothing is left in
+ * the barrier protocol (no loads, no stores), so nothing is left in
  * flight and the context stays usable; the per-instance records then carry
  * FTSP2_E_TIMEOUT (returned with FTSP2_SYNC) and the outputs are not valid.
  * The next call starts from a cleared status word.  (No counterpart in the

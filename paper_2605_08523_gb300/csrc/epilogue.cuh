@@ -48,8 +48,8 @@ __device__ __forceinline__ void store_partial(const LayerArgs& a, int inst, int 
 }
 
 struct EpiCtx {
-    int n, P, chain, kind, flip, last, next_fmt;
-    float mul;            // multiplier of the product: a_k, times 2^(-2 e_k) for scaled FP16 operands
+    int n, P, chain, kind, flip, last;
+    float mul;            // multiplier of the product: a_k
     size_t slab;          // b * P * P
     int64_t doff;         // D offset
     DevLayer L;
@@ -187,8 +187,7 @@ __device__ __forceinline__ void epi_segment_max(const LayerArgs& a, const EpiCtx
     }
 }
 
-// `scaled_in`: the products were formed from power-of-two scaled FP16 operands.
-__device__ __forceinline__ void make_ctx(const LayerArgs& a, const Tile& t, int k, EpiCtx& e, bool scaled_in) {
+__device__ __forceinline__ void make_ctx(const LayerArgs& a, const Tile& t, int k, EpiCtx& e) {
     const ftsp2_instance in = a.inst[t.inst];
     const ftsp2_rescale_rec& rec = a.rec[t.inst];
     const DevModel& M = a.models[rec.model];
@@ -198,12 +197,11 @@ __device__ __forceinline__ void make_ctx(const LayerArgs& a, const Tile& t, int 
     e.kind = a.chain_kind[t.chain];
     e.flip = rec.flip;
     e.last = a.last;
-    e.next_fmt = a.next_fmt;
     e.slab = (size_t)t.inst * a.P * a.P;
     e.doff = in.offset;
     e.L = a.layers[(e.kind == CHAIN_ENTROPY ? M.offS : M.off) + k];
     e.cdiag = rec.flip ? 1.0 - M.f0 : M.f0;
-    e.mul = scaled_in ? e.L.acc_mul : e.L.a;
+    e.mul = e.L.a;
 }
 
 }  // namespace ftsp2

@@ -470,8 +470,8 @@ static ftsp2_status plan(const ftsp2_instance* inst, int nb, int mode, int want,
     const bool simt_main = mode == FTSP2_FP32;
     const bool refine = !simt_main && refine_layers(flags) > 0;
     // tiles of each shape; the tile of a call's main table is that of its shape
-    // (128 x 128 in FP32 mode), a second table of 128 x 128 tiles serves
-    // single-CTA layers and FP32 refinement layers
+    // (128 x 128 in FP32 mode), a second table of 128 x 128 tiles serves the FP32
+    // refinement layers of calls on the other shapes
     long long nt[kShapes] = {};
     for (int b = 0; b < nb; ++b)
         for (int sh = 0; sh < kShapes; ++sh) nt[sh] += host_tiles_of(inst[b].n, tc_block_m(sh), tc_block_n(sh));

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kSThreads, 4) layer_simt_kernel(const __grid_c
         for (int j = 0; j < 4; ++j) sm[(ty * 8 + i) * kSPitch + tx * 4 + j] = acc[i][j];
     __syncthreads();
     EpiCtx e;
-    make_ctx(a, tl, k, e, false);
+    make_ctx(a, tl, k, e);
     double tr = 0.0, sq = 0.0;
     // 32 x 8 blocks of the quadrant, lane = row
 #pragma unroll 1

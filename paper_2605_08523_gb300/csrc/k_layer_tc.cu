@@ -102,7 +102,10 @@
 // FTSP2_E_TIMEOUT in the status word of the call; from then on every role of
 // every CTA that sees the failure runs the rest of its work items in skip
 // mode: the same barrier arrivals, waits and commits in the same order, but no
-// TMA loads, MMAs or epilogue stores.  Every barrier phase therefore still
+// TMA loads and no epilogue stores.  layer_tc_kernel's MMAs still run, on whatever
+// their stage holds (one CTA of a pair may skip while its peer loads): they write
+// only TMEM, their sums are not stored, and their commits complete the phases as
+// usual; layer_defer_kernel leaves them out.  Every barrier phase therefore still
 // completes and nothing is in flight when the work list ends; the MMA issuer
 // also waits for a last commit of its own before the CTAs free TMEM.  A
 // pipeline wait that runs out twice (a broken protocol, not expected) leaves
@@ -260,8 +263,8 @@ __device__ __forceinline__ void record_timeout(const LayerArgs& a) { atomicCAS(a
 
 // Wait on a pipeline mbarrier phase.  A failure elsewhere never ends such a
 // wait: after a failure every role keeps the barrier protocol of its work list
-// (arrivals and commits in the usual order, without loads, MMAs or stores), so
-// every phase still completes.  The wait gives up only on its own clock: after
+// (arrivals and commits in the usual order, without loads or stores), so every
+// phase still completes.  The wait gives up only on its own clock: after
 // a.wait_ns it records FTSP2_E_TIMEOUT (the call has failed), and after twice
 // that it returns false, which only a broken protocol can cause; the caller
 // then leaves its loop and the kernel drains before it frees TMEM.
@@ -422,57 +425,30 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// ----------------------------------------------------------------------------------
-// Split formats of the next layer's operands (planes of 2- or 4-byte
-// elements); the stores themselves are in epi_dgroup_next.
-// ----------------------------------------------------------------------------------
+// Split formats of the next layer's operands: planes, bytes of an element.
 template <int FMT>
 struct OpFmtT;
 template <>
 struct OpFmtT<OP_F16X2> {
     static constexpr int NPL = 2, ESZ = 2;
-    __device__ static void split(float z, uint32_t* o) {
-        const __half h = __float2half_rn(z);
-        const __half l = __float2half_rn(z - __half2float(h));
-        o[0] = __half_as_ushort(h);
-        o[1] = __half_as_ushort(l);
-    }
 };
 template <>
 struct OpFmtT<OP_BF16X3> {
     static constexpr int NPL = 3, ESZ = 2;
-    __device__ static void split(float z, uint32_t* o) {
-        const __nv_bfloat16 b0 = __float2bfloat16_rn(z);
-        const float r1 = z - __bfloat162float(b0);
-        const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 b2 = __float2bfloat16_rn(r1 - __bfloat162float(b1));
-        o[0] = __bfloat16_as_ushort(b0);
-        o[1] = __bfloat16_as_ushort(b1);
-        o[2] = __bfloat16_as_ushort(b2);
-    }
 };
 template <>
 struct OpFmtT<OP_TF32X3> {
     static constexpr int NPL = 2, ESZ = 4;
-    __device__ static void split(float z, uint32_t* o) {
-        uint32_t hb;
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hb) : "f"(z));
-        o[0] = hb;
-        // the tensor core reads only the TF32 bits of the low part: round it
-        // to TF32 (unbiased) instead of letting the low 13 bits be cut
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(o[1]) : "f"(z - __uint_as_float(hb)));
-    }
 };
 template <>
 struct OpFmtT<OP_F32> {
     static constexpr int NPL = 1, ESZ = 4;
-    __device__ static void split(float z, uint32_t* o) { o[0] = __float_as_uint(z); }
 };
 
 constexpr int kLastLayer = -1;
 
-// The same, past the L1 (no reuse, and in multi-layer launches other CTAs write
-// it) and in program order with the waits around it.
+// The 8 state values of a row past the L1 (no reuse, and in multi-layer launches
+// other CTAs write them) and in program order with the waits around it.
 __device__ __forceinline__ void ld_state8(const float* S, float* x) {
     asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
@@ -622,9 +598,10 @@ __device__ __forceinline__ void load16(const LayerArgs& a, const float* Zs, int 
     }
 }
 
-// The planes of a split are formed one after the other from what the planes
-// before left of z (the steps of OpFmtT<FMT>::split): 32 columns of one plane as
-// packed words (two columns a word for the 16-bit formats).
+// The planes of a split are formed one after the other, each rounded to nearest
+// from what the planes before left of z (TF32X3: the low part too, since the tensor
+// core would cut its low 13 bits): 32 columns of one plane as packed words (two
+// columns a word for the 16-bit formats).
 template <int FMT>
 struct PlaneWords {
     static constexpr int ESZ = OpFmtT<FMT>::ESZ, N = 8 * ESZ;
@@ -839,7 +816,7 @@ __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c
 }
 
 // Last layer on the warp's 32 x COLS block, 8 columns at a time, the state loaded
-// one 16-column group ahead as in epi_block: G = A + d Z + g xh with
+// one 32-column block ahead: G = A + d Z + g xh with
 // xh = mul v + bp Z (Eq. mlsp2: A_L + Z_L, A_L = A_{L-1} + d Z_{L-1},
 // Z_L = a v + b' Z_{L-1}; Skip-SP2: A_L + gamma_L x_L), then D = G + f0 I (or
 // (1 - f0) I - G when flipped) at (r, c) and (c, r), and the sums of the
@@ -1036,7 +1013,7 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
     __shared__ __align__(8) uint64_t drain_bar;
     __shared__ uint32_t tmem_slot;
     // skip mode: set once this CTA has seen the call fail; the roles then keep
-    // the barrier protocol of their work items without loads, MMAs or stores
+    // the barrier protocol of their work items without loads or stores
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1208,7 +1185,8 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
                     const uint32_t fb = full0 + 8u * stage;
                     if (skip) {
                         // the stage's arrival without data: the phase completes
-                        // with the peer's loads (if any) and no MMA reads it
+                        // with the peer's loads (if any), and the sums of the MMAs
+                        // that read it are not used
                         if constexpr (PAIR) remote_arrive(fb);
                         else local_arrive(fb);
                     } else {

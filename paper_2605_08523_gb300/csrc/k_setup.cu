@@ -7,7 +7,8 @@
 //   init       -- (a2) layer-0 state Z_0 = scale (mu I - H) (Eq. H0, centred),
 //                 accumulators, first-layer tensor-core operands
 //   finalize   -- (a4, a6) Tr D, ||D||_F^2 (Eq. tr(D^2)) and S (Eq. entropy
-//                 expansion-s) from per-tile FP64 partial sums, in a fixed order
+//                 expansion-s) from FP64 partial sums per 32 x 64 block, in a
+//                 fixed order
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
