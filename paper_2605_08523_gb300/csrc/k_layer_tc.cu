@@ -56,14 +56,14 @@
 //                an instruction every eleven clocks), so FP16X2 operands of
 //                128-column tiles have 16 warps of 32 columns (96 registers) and
 //                256-column tiles 16 warps of 64; the others have 8 warps of 64
-//                columns (168 registers), 128 at the last layer: there the wider
-//                formats' planes spill in 96.  8 -> 16 warps, FP16X2: n = 256
+//                columns (168 registers): the wider formats' planes spill in 96.  8 -> 16 warps, FP16X2: n = 256
 //                277 -> 261 us, 60 fragments 411 -> 380, ragged batch 22.8 ->
 //                22.1 ms, n = 1501 unchanged; BF16X3 and TF32X3 on 128 columns
 //                0.7 % slower at n = 1024 and 2048.  256 x 256 tiles, inline, 8 ->
 //                16 warps with the state 16 columns ahead: n = 2200 TF32X3
 //                (density) 2173 -> 2038 us, n = 2700 FP16X2 1526 -> 1456, n = 2816
-//                FP16X2 (density + entropy) 2716 -> 2546.
+//                FP16X2 (density + entropy) 2716 -> 2546; their last layer at n =
+//                4096 440 -> 332.
 //   last warp  : context warp (below)
 // The loops of warps 0 and 1 run on the whole warp with one elected lane issuing:
 // their values are then uniform, and a copy or an MMA takes no moves from vector
@@ -161,7 +161,7 @@ constexpr int kCtaRows = 128;
 template <int OUTFMT, int SHAPE>
 constexpr int epi_warps() {
     if (SHAPE == SHAPE_SINGLE64) return OUTFMT == -1 ? 4 : 8;     // last layer: a 32 x 64 block of partial sums a warp
-    return OUTFMT != -1 && (OUTFMT == OP_F16X2 || SHAPE == SHAPE_PAIR) ? 16 : 8;
+    return SHAPE == SHAPE_PAIR || OUTFMT == OP_F16X2 ? 16 : 8;
 }
 template <int OUTFMT, int SHAPE>
 constexpr int tc_threads() { return 32 * (2 + epi_warps<OUTFMT, SHAPE>() + 1); }
@@ -815,8 +815,7 @@ __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c
     }
 }
 
-// Last layer on the warp's 32 x COLS block, 8 columns at a time, the state loaded
-// one 32-column block ahead: G = A + d Z + g xh with
+// Last layer on the warp's 32 x COLS block, 8 columns at a time: G = A + d Z + g xh with
 // xh = mul v + bp Z (Eq. mlsp2: A_L + Z_L, A_L = A_{L-1} + d Z_{L-1},
 // Z_L = a v + b' Z_{L-1}; Skip-SP2: A_L + gamma_L x_L), then D = G + f0 I (or
 // (1 - f0) I - G when flipped) at (r, c) and (c, r), and the sums of the
@@ -832,8 +831,9 @@ struct LastSums {
     double tr, sq;
     float lo;
 };
-__device__ __forceinline__ void epi_last32(const LayerArgs& a, const ItemCtx& c, int R0, int lane, int c0,
-                                           const float (&v)[32], const State32& s, LastSums& b) {
+template <int COLS>
+__device__ __forceinline__ void epi_last(const LayerArgs& a, const ItemCtx& c, int R0, int lane, int c0,
+                                         const float* v, const float* zs, const float* xs, LastSums& b) {
     const int n = c.n, r = R0 + lane;
     const float mul = c.mul, bp = c.bp, d = c.d, g1 = c.g, cdiag = c.cdiag;
     const bool flip = c.flip != 0, dout = c.dout != 0;
@@ -843,7 +843,7 @@ __device__ __forceinline__ void epi_last32(const LayerArgs& a, const ItemCtx& c,
     double tr = b.tr, sq = b.sq;
     float lo = b.lo;
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
+    for (int h = 0; h < COLS / 8; ++h) {
         const int cc0 = c0 + 8 * h;
         if (cc0 >= n) break;
         float dv[8];
@@ -851,7 +851,7 @@ __device__ __forceinline__ void epi_last32(const LayerArgs& a, const ItemCtx& c,
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int cc = cc0 + u;
-            const float z = s.z[h >> 1][8 * (h & 1) + u], x = s.x[h >> 1][8 * (h & 1) + u];
+            const float z = zs[8 * h + u], x = xs[8 * h + u];
             const float g = fmaf(g1, fmaf(mul, v[8 * h + u], bp * z), fmaf(d, z, x));
             const bool diag = r == cc;
             if (flip) dv[u] = (diag ? cdiag : 0.f) - g;
@@ -1515,9 +1515,28 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
                     lb.tr = lb.sq = 0.0;
                     lb.lo = 0.f;
                 };
-                if (live && work) {
+                if constexpr (HOLD) {
+                    if (live && work) {
+                        // a warp's 32 x 64 block, 8 columns at a time: the registers of
+                        // sixteen warps hold no more without spills (16 columns 359 us a
+                        // layer of n = 4096, D + S; with the next 16 ahead 365; 332 so)
+                        const uint32_t tfin = tlane + (uint32_t)(buf * TN);
+                        const float* Zg = c.Z + state_off(a.P, R0 + lane, C0 + cb0);
+#pragma unroll 2
+                        for (int cb = cb0; cb < cb1 && C0 + cb < n; cb += 8, Zg += 256) {
+                            float v[8], z[8], x[8];
+                            tmem_ld8(tfin + cb, reinterpret_cast<uint32_t*>(v));
+                            ld_state8(Zg, z);
+                            ld_state8(Zg + a.plane_elems, x);
+                            tmem_wait_ld();
+                            epi_last<8>(a, c, R0, lane, C0 + cb, v, z, x, lb);
+                            __syncwarp();
+                        }
+                        flush(C0 + cb0);
+                    }
+                } else if (live && work) {
                     blocks([&](int cb, float (&v)[32], State32& s) {
-                        epi_last32(a, c, R0, lane, C0 + cb, v, s, lb);
+                        epi_last<32>(a, c, R0, lane, C0 + cb, v, s.z[0], s.x[0], lb);
                         if (next_of(cb) >= 0) {
                             load16(a, c.Z, n, R0, R0 + lane, next_of(cb), s.z[0], s.x[0]);
                             load16(a, c.Z, n, R0, R0 + lane, next_of(cb) + 16, s.z[1], s.x[1]);
