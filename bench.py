@@ -344,15 +344,15 @@ def plain_fp32_recursion(Hd, mu, kT, theta, beta0, mu0, alpha, emin, emax, theta
 # bytes) of one ragged-batch layer launch with every instance active, from an
 # ncu capture of that launch at that code hash
 MEASURED_RAGGED_TRAFFIC = {
-    # 512-instance ragged batch, global layer 35 of 44: 1.78 GB read + 1.55 GB
-    # written in 0.937 ms
-    ("fp16x2", 512, "215c1725bf044bed"): (3.33e9, 3.285e9),
+    # 512-instance ragged batch, global layer 35 of 44: 1.74 GB read + 1.60 GB
+    # written in 0.804 ms
+    ("fp16x2", 512, "2eb3cb0943b4c191"): (3.34e9, 3.285e9),
 }
 
 MEASURED_TRAFFIC = {
-    # n = 8192 long-range lattice, FP16X2 main layer (layer_tc_kernel<FP16X2,
-    # FP16X2, pair, deferred>): 3.22 GB read + 1.04 GB written per launch
-    ("fp16x2", 8192, "215c1725bf044bed"): 4.26e9,
+    # n = 8192 long-range lattice, FP16X2 main layer (layer_defer_kernel<FP16X2,
+    # FP16X2>): 3.48 GB read + 1.06 GB written per launch
+    ("fp16x2", 8192, "2eb3cb0943b4c191"): 4.54e9,
 }
 
 
