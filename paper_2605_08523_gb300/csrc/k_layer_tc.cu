@@ -744,13 +744,13 @@ struct State {
 using State32 = State<2>;
 
 // One 32 x 32 block: v holds the sums S of the lane's row, s the state of its 32
-// columns (H = 2) or of the first 16 (H = 1).  fetch(h) follows the use of half h:
-// it loads that half of the next block (H = 2), or the second half of this block
-// (h = 0) and the first one of the next (h = 1).
+// columns (H = 2) or of the first 16 (H = 1).  After the use of half h the same half
+// of the next block (at column c_next; -1: none) is loaded (H = 2), or fetch(h) loads
+// the second half of this block (h = 0) and the first one of the next (h = 1).
 template <int FMT, bool CAN_RESIDE, int H, class Fetch>
 __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c, const CUtensorMap* wmaps, Stager& st,
                                             int R0, int c0, uint32_t tstate, bool from_tmem, bool to_tmem,
-                                            float (&v)[32], State<H>& s, Fetch&& fetch) {
+                                            float (&v)[32], State<H>& s, int c_next, Fetch&& fetch) {
     constexpr int NPL = OpFmtT<FMT>::NPL;
     const int n = c.n, r = R0 + st.lane;
     const float mul = c.mul, bp = c.bp, d = c.d;
@@ -793,7 +793,11 @@ __device__ __forceinline__ void epi_block32(const LayerArgs& a, const ItemCtx& c
                 }
             }
         }
-        fetch(h);
+        if constexpr (H == 2) {
+            if (!from_tmem && c_next >= 0) load16(a, c.Z, n, R0, r, c_next + 16 * h, s.z[h], s.x[h]);
+        } else {
+            fetch(h);
+        }
     }
     if (!(R0 + 31 < n && c0 + 31 < n)) {
         // zeros in the padding
@@ -1483,17 +1487,12 @@ __global__ void __launch_bounds__((tc_threads<OUTFMT, SHAPE>()), 1)
                 if (live && work) {
                     const CUtensorMap* const wm = (c.maps ? wmaps1 : wmaps0).w[c.chain];
                     blocks([&](int cb, float (&v)[32], State<AH>& s) {
+                        const int cn = next_of(cb);
                         epi_block32<OUTFMT, CAN_RESIDE, AH>(
-                            a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem, to_tmem, v, s, [&](int h) {
-                                const int cn = EPI_COLS > 32 ? next_of(cb) : -1;
+                            a, c, wm, st, R0, C0 + cb, tlane + kStateZ + cb, from_tmem, to_tmem, v, s, cn, [&](int h) {
                                 if (from_tmem) return;
-                                if constexpr (AH == 2) {
-                                    if (cn >= 0) load16(a, c.Z, n, R0, R0 + lane, cn + 16 * h, s.z[h], s.x[h]);
-                                } else if (h == 0) {
-                                    load16(a, c.Z, n, R0, R0 + lane, C0 + cb + 16, s.z[0], s.x[0]);
-                                } else if (cn >= 0) {
-                                    load16(a, c.Z, n, R0, R0 + lane, cn, s.z[0], s.x[0]);
-                                }
+                                if (h == 0) load16(a, c.Z, n, R0, R0 + lane, C0 + cb + 16, s.z[0], s.x[0]);
+                                else if (EPI_COLS > 32 && cn >= 0) load16(a, c.Z, n, R0, R0 + lane, cn, s.z[0], s.x[0]);
                             });
                     });
                     if (CAN_RESIDE && to_tmem) tmem_wait_st();
@@ -1927,7 +1926,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                         if (next) issue(en, h, h);
                     };
                     take(0);
-                    epi_block32<OUTFMT, false>(a, c, wm, st, d.R0, d.c0, 0u, false, false, v, s, [&](int h) {
+                    epi_block32<OUTFMT, false>(a, c, wm, st, d.R0, d.c0, 0u, false, false, v, s, -1, [&](int h) {
                         if (h == 0) take(1);
                     });
                     e = en;
@@ -2072,7 +2071,7 @@ __global__ void __launch_bounds__(kDeferThreads, 1)
                     load16(a, c.Z, c.n, R0, R0 + lane, c0, s.z[0], s.x[0]);
                     tmem_ld32(tfin + cb, reinterpret_cast<uint32_t*>(v));
                     tmem_wait_ld();
-                    epi_block32<OUTFMT, false>(a, c, wm, st, R0, c0, 0u, false, false, v, s, [&](int h) {
+                    epi_block32<OUTFMT, false>(a, c, wm, st, R0, c0, 0u, false, false, v, s, -1, [&](int h) {
                         if (h == 0) load16(a, c.Z, c.n, R0, R0 + lane, c0 + 16, s.z[0], s.x[0]);
                     });
                 }
